@@ -17,7 +17,7 @@
 #include "eik.h"
 #include "eik_host.h"
 #include "eik_internal.cuh"
-#include "eik_march.cuh"
+#include "eik_march8.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -100,16 +100,19 @@ __device__ __forceinline__ void batch_bounds_ahead(const LoopParams<T>& P, int k
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) {
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_loop(LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
     __shared__ LoopState s_state[kWarps];
+    __shared__ MarchAcc s_acc[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
+    QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
     LoopState& L = s_state[warp];              // the loop's bookkeeping, kept out of registers
     Ctrl* C = P.ctrl;
     if (threadIdx.x == 0) s_arrived = 0;
+    init_queue_smem(SQ[warp], lane);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned long long t0 = globaltimer();
@@ -117,7 +120,8 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
         C->t_restart = t0;
     }
     if (lane == 0) L.claim = -1;
-    MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+    MarchAcc& A = s_acc[warp];
+    if (lane == 0) reset_acc(A);
     bool any = false;
     for (;;) {
         const int k = __ldcg(&C->k);
@@ -128,6 +132,8 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
         if (!cta_go(C, true, lane, &s_arrived)) return;
         {
             const int n = __ldcg(&C->gcount[s]);
+            MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+            bool grouped = false;
             for (;;) {
                 __syncthreads();
                 if (threadIdx.x == 0) {
@@ -140,7 +146,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
                 if (g < 0) break;
                 const int sv = __ldg(P.gsolve + g);
                 const SolveDesc D = P.solves[sv];
-                const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 2u};
+                const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 2u, D.div_x, D.div_xy};
                 const int gl = g - D.goff;
                 const int gx = gl % D.GX, gy = (gl / D.GX) % D.GY, gz = gl / (D.GX * D.GY);
                 const int bx = 2 * gx + (warp & 1), by = 2 * gy + ((warp >> 1) & 1), bz = 2 * gz + (warp >> 2);
@@ -155,10 +161,14 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
                     if (warp & 4) gmask |= 16u;
                     else if (bz + 1 < D.BZ) gmask |= 32u;
                 }
-                march<T, true>(P, G, SW, warp, b, gmask, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
+                march_group<T>(P, G, SW, warp, b, gmask, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
                                pick<T>(P.window, P.window_f), lane, acc, early_k);
                 if (threadIdx.x == 0) atomicMax(P.last_k + sv, k);
-                any = true;
+                grouped = true;
+            }
+            if (grouped) {
+                flush_acc(C, acc, lane);
+                init_queue_smem(SQ[warp], lane);              // (the groups' tiles overlay it)
             }
         }
         // ---- 8^3 blocks, one warp per brick: this restart's list, then -- once
@@ -188,7 +198,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
                 i = __shfl_sync(kFull, i, 0);
                 if (i >= 0) b = take_entry(P.list[s], i, false, 0, lane);
                 if (b < 0) {
-                    if (any) flush_acc(C, acc, lane);
+                    if (any) flush_acc8(C, A, lane);
                     any = false;
                     unsigned gen;
                     if (barrier_arrive(C, lane, &gen)) {
@@ -215,7 +225,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
                 }
                 if (b >= 0) {
                     const SolveDesc D = P.solves[__ldg(P.bsolve + b)];
-                    const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u};
+                    const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u, D.div_x, D.div_xy};
                     if (!wait_ready(P, G, b, k, lane)) b = -2;
                 }
                 if (b == -2) {
@@ -246,9 +256,9 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_batch_loop(LoopParams<T> P) 
             __syncwarp();
             const int sv = __ldg(P.bsolve + b);
             const SolveDesc D = P.solves[sv];
-            const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u};
-            march<T, false>(P, G, SW, warp, b, 0u, kk, batch_bound(P, sv, kk - 1), batch_bound(P, sv, kk), true,
-                            pick<T>(P.window, P.window_f), lane, acc, early_k || kk > k);
+            const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u, D.div_x, D.div_xy};
+            march8<T>(P, G, SQ[warp], A, b, kk, batch_bound(P, sv, kk - 1), batch_bound(P, sv, kk), true,
+                            pick<T>(P.window, P.window_f), lane, early_k || kk > k);
             if (lane == 0) atomicMax(P.last_k + sv, kk);
             any = true;
         }
@@ -292,7 +302,7 @@ __global__ void k_owner(int32_t* __restrict__ tab, int64_t n, const int32_t* __r
 
 template <typename T>
 size_t batch_smem_bytes() {
-    return sizeof(WarpSmem<T>) * kWarps;
+    return std::max(sizeof(WarpSmem<T>), sizeof(QueueSmem<T>)) * kWarps;
 }
 
 template <typename T>
@@ -603,6 +613,8 @@ eik_status batch_queue(eik_batch* b, const std::vector<eik_batch_tile>& tiles, i
         d.goff = G.goff;
         d.mode = tiles[i].block_dim;
         d.stride = tiles[i].stride;
+        d.div_x = eikg::make_fastdiv(d.BX);
+        d.div_xy = eikg::make_fastdiv(static_cast<int64_t>(d.BX) * d.BY);
         if (d.mode == 16) genq.insert(genq.end(), G.genq.begin(), G.genq.end());
         else enq.insert(enq.end(), G.enq.begin(), G.enq.end());
     }
@@ -661,6 +673,7 @@ eik_status batch_queue(eik_batch* b, const std::vector<eik_batch_tile>& tiles, i
         L.window = P.window;
         L.window_f = static_cast<float>(P.window);
         L.fallback_tau = P.fallback_tau;
+        L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.width = INFINITY;                    // full solves
         L.wait_limit = eikg::kWaitPolls;

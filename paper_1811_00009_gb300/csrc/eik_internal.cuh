@@ -4,7 +4,8 @@
 // of its grids, see SolveDesc):
 //   bricks of 8x8x8 nodes, brick b = (bz*BY + by)*BX + bx, node p = (z*8 + y)*8 + x
 //   inside a brick; a ragged last brick per axis is padded with barrier nodes.
-//   rr[b][512]          h/F (+inf: barrier or padding, -1: fixed source node)
+//   rr[b][512]          h/F (-inf: a node that is never solved: barrier, padding,
+//                       a fixed source node during a solve)
 //   slot[b][2][640]     two copies of the brick's psi: 512 interior values,
 //                       then its x = 0 and x = 7 faces (64 each, index z*8+y)
 //                       stored contiguously for the neighbours' ghost reads
@@ -118,6 +119,24 @@ struct FaceRec {
     int32_t pad;
 };
 
+// Division by a launch constant d >= 1 of n < 2^31 (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994): n / d =
+// (n * m) >> s with s = 31 + ceil(log2 d), m = ceil(2^s / d).  A march splits
+// its brick index twice; the hardware has no integer divider.
+struct FastDiv {
+    uint32_t m;
+    int32_t s;
+};
+__host__ inline FastDiv make_fastdiv(int64_t d) {
+    int l = 0;
+    while ((int64_t(1) << l) < d) ++l;
+    const unsigned long long p = 1ull << (31 + l);
+    return FastDiv{static_cast<uint32_t>((p + static_cast<unsigned long long>(d) - 1) / static_cast<unsigned long long>(d)), 31 + l};
+}
+__host__ __device__ inline int32_t fast_div(int32_t n, FastDiv d) {
+    return static_cast<int32_t>((static_cast<unsigned long long>(static_cast<uint32_t>(n)) * d.m) >> d.s);
+}
+
 // One grid of a batched launch: its place in the launch's brick and group
 // index spaces, its block edge and its stride (bound of restart k = k*stride).
 struct SolveDesc {
@@ -128,12 +147,14 @@ struct SolveDesc {
     int32_t mode;              // block edge: 8 (one warp per brick) or 16 (one CTA per group)
     int32_t pad;
     double stride;
+    FastDiv div_x, div_xy;     // by BX and BX*BY
 };
 
 template <typename T>
 struct LoopParams {
     int32_t nx, ny, nz;
     int32_t BX, BY, BZ;
+    FastDiv div_x, div_xy;     // by BX and BX*BY
     int64_t nbricks;
     int64_t ngroups;
     T* slot;
@@ -158,6 +179,7 @@ struct LoopParams {
     double window;             // omega: acceptance window = omega * min(h/F) over the brick
     float window_f;            // omega in single precision (FP32 marches compute the window in float)
     double fallback_tau;       // FP32: double-precision root when D < tau * k * r^2
+    float tau_f;               // the same in single precision
     int64_t max_restarts;
     long long wait_limit;      // polls before a wait (barrier, list entry, neighbour march) gives up
     int32_t sched;             // 0 fixed, 1 learned, 2 seeded random (exploration data)

@@ -7,9 +7,10 @@
 // the start of the next march (see eik_internal.cuh for the double-copy
 // layout that makes this race-free, the argument of Sec. 2.7).
 #include "eik_internal.cuh"
-#include "eik_march.cuh"
+#include "eik_march8.cuh"
 #include "eik_mlp.cuh"
 
+#include <algorithm>
 #include <cfloat>
 #include <cstdint>
 
@@ -75,7 +76,7 @@ __device__ __forceinline__ void next_restart_of(const LoopParams<T>& P, const Ct
 template <typename T>
 __device__ void restart_end(const LoopParams<T>& P, int lane, float* scratch) {
     static_assert(kHid == 32, "one hidden unit per lane");
-    static_assert(sizeof(WarpSmem<T>) >= (kHid * (kIn + 1) + (kHid + kAct) * (kHid + 1)) * sizeof(float),
+    static_assert(sizeof(QueueSmem<T>) >= (kHid * (kIn + 1) + (kHid + kAct) * (kHid + 1)) * sizeof(float),
                   "the staged weights fit the warp's tile");
     __shared__ float s_x[kIn];
     __shared__ float s_h1[kHid];
@@ -229,29 +230,34 @@ __device__ __noinline__ bool groups_from_bricks(Ctrl* C, const int32_t* list, in
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P) {
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart_loop(LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
     __shared__ LoopState s_state[kWarps];
+    __shared__ MarchAcc s_acc[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
+    QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
     LoopState& L = s_state[warp];              // the loop's bookkeeping, kept out of registers
     Ctrl* C = P.ctrl;
     if (threadIdx.x == 0) s_arrived = 0;
+    init_queue_smem(SQ[warp], lane);
     __syncthreads();
     // Work lists the marches fill: the brick list, and for fixed 16^3 blocks
     // the group list too.  Under a learned or random schedule a 16^3 restart
     // builds its group list from its brick list when it starts (such restarts
     // are rare, and every enqueue would otherwise pay for the group list).
-    const Geo G{P.BX, P.BY, P.BZ, 0, P.GX, P.GY, 0, (P.groups && P.sched == 0) ? 3u : 1u};
+    const Geo G{P.BX, P.BY, P.BZ, 0, P.GX, P.GY, 0, (P.groups && P.sched == 0) ? 3u : 1u,
+                P.div_x, P.div_xy};
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned long long t0 = globaltimer();
         C->t_begin = t0;
         C->t_restart = t0;
     }
     if (lane == 0) L.claim = -1;
-    MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+    MarchAcc& A = s_acc[warp];
+    if (lane == 0) reset_acc(A);
     bool any = false;                          // acc holds something to flush
     for (;;) {
         const int k = __ldcg(&C->k);
@@ -283,6 +289,8 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P
                                                P.glist[s], s, k, P.BX, P.BY, P.GX, P.GY, lane, P.wait_limit);
             if (!cta_go(C, ok, lane, &s_arrived)) return;
             // one CTA per group of 2x2x2 bricks
+            MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+            bool grouped = false;
             const int n = __ldcg(&C->gcount[s]);
             for (;;) {
                 __syncthreads();
@@ -307,10 +315,12 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P
                     if (warp & 4) gmask |= 16u;
                     else if (bz + 1 < P.BZ) gmask |= 32u;
                 }
-                march<T, true>(P, G, SW, warp, b, gmask, k, pick<T>(L.bprev, L.bprev_f), pick<T>(L.bound, L.bound_f),
+                march_group<T>(P, G, SW, warp, b, gmask, k, pick<T>(L.bprev, L.bprev_f), pick<T>(L.bound, L.bound_f),
                                L.grow != 0, pick<T>(P.window, P.window_f), lane, acc, L.early != 0);
-                any = true;
+                grouped = true;
             }
+            if (grouped) flush_acc(C, acc, lane);
+            init_queue_smem(SQ[warp], lane);          // (the groups' tiles overlay it)
         }
         // One warp per 8^3 brick: this restart's list, then -- once arrived at
         // the barrier -- restart k+1's bricks whose neighbourhood has finished
@@ -339,11 +349,12 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P
                     if (pf >= P.nbricks) pf = -1;
                 }
                 if (b < 0) {
-                    if (any) flush_acc(C, acc, lane);
+                    if (any) flush_acc8(C, A, lane);
                     any = false;
                     unsigned gen;
                     if (barrier_arrive(C, lane, &gen)) {
-                        restart_end<T>(P, lane, reinterpret_cast<float*>(SW + warp));
+                        restart_end<T>(P, lane, reinterpret_cast<float*>(SQ + warp));
+                        init_queue_smem(SQ[warp], lane);      // (the weights were staged there)
                         barrier_release(C, lane, gen);
                         break;
                     }
@@ -391,10 +402,10 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P
             }
             __syncwarp();
             const bool ahead = kk > k;
-            march<T, false>(P, G, SW, warp, b, 0u, kk,
+            march8<T>(P, G, SQ[warp], A, b, kk,
                             ahead ? pick<T>(L.bound, L.bound_f) : pick<T>(L.bprev, L.bprev_f),
                             ahead ? pick<T>(L.next_bound, L.next_f) : pick<T>(L.bound, L.bound_f),
-                            (ahead ? L.grow_next : L.grow) != 0, pick<T>(P.window, P.window_f), lane, acc,
+                            (ahead ? L.grow_next : L.grow) != 0, pick<T>(P.window, P.window_f), lane,
                             L.early != 0 || ahead, pf);
             any = true;
         }
@@ -402,7 +413,9 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_restart_loop(LoopParams<T> P
     }
 }
 
-// F (x fastest) -> h/F in brick layout; flags negative, NaN or infinite speeds.
+// F (x fastest) -> h/F in brick layout (-inf where a node is never solved: F = 0,
+// padding, or h/F outside the positive range of T, so that marches need no test);
+// flags negative, NaN or infinite speeds.
 template <typename T>
 __global__ void k_layout_speed(const T* __restrict__ F, T* __restrict__ rr, int nx, int ny, int nz, int BX,
                                int BY, int64_t nbricks, double h, int* err, int seq) {
@@ -412,7 +425,7 @@ __global__ void k_layout_speed(const T* __restrict__ F, T* __restrict__ rr, int 
     const T hT = static_cast<T>(h);
     // one block per row (k, j) of the padded brick grid at a time, its threads
     // along x: each warp reads 128 contiguous bytes of F and writes 32-byte runs
-    // of four bricks; padding nodes get +inf
+    // of four bricks
     const int px = BX * 8, py = BY * 8;
     const int64_t rows = (nbricks / (static_cast<int64_t>(BX) * BY)) * 8 * py;
     int bad = 0;
@@ -422,11 +435,12 @@ __global__ void k_layout_speed(const T* __restrict__ F, T* __restrict__ rr, int 
         const int64_t frow = inrow ? (static_cast<int64_t>(k) * ny + j) * nx : 0;
         T* out = rr + ((static_cast<int64_t>(k >> 3) * BY + (j >> 3)) * BX) * kBrick + ((k & 7) * 8 + (j & 7)) * 8;
         for (int i = threadIdx.x; i < px; i += blockDim.x) {
-            T v = INF;
+            T v = -INF;
             if (inrow && i < nx) {
                 const T f = __ldg(F + frow + i);
                 if (!(f >= 0) || !(f < INF)) bad = 1;
                 else if (f > 0) v = hT / f;
+                if (!(v > 0) || !(v < INF)) v = -INF;
             }
             __stcs(out + (i >> 3) * kBrick + (i & 7), v);
         }
@@ -464,7 +478,7 @@ __global__ void k_init_sources(int nfix, const int32_t* __restrict__ fix_b, cons
         if (base < nfix) {
             const int64_t g = static_cast<int64_t>(fix_b[base]) * kBrick + fix_p[base];
             saved_r[base] = rr[g];
-            rr[g] = static_cast<T>(-1);
+            rr[g] = -INF;
         }
         if (base < nenq) {
             list1[base] = enq[base];
@@ -528,16 +542,17 @@ __global__ void k_layout_speed_x4(const float* __restrict__ F, float* __restrict
         const int64_t frow = inrow ? (static_cast<int64_t>(k) * ny + j) * nx : 0;
         float* out = rr + ((static_cast<int64_t>(k >> 3) * BY + (j >> 3)) * BX) * kBrick + ((k & 7) * 8 + (j & 7)) * 8;
         for (int i = 4 * threadIdx.x; i < px; i += 4 * blockDim.x) {
-            float4 v = make_float4(INF, INF, INF, INF);
+            float4 v = make_float4(-INF, -INF, -INF, -INF);
             if (inrow && i < nx) {
                 const float4 f = __ldg(reinterpret_cast<const float4*>(F + frow + i));
                 const float fq[4] = {f.x, f.y, f.z, f.w};
                 float vq[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    vq[e] = INF;
+                    vq[e] = -INF;
                     if (!(fq[e] >= 0.0f) || !(fq[e] < INF)) bad = 1;
                     else if (fq[e] > 0.0f) vq[e] = hT / fq[e];
+                    if (!(vq[e] > 0.0f) || !(vq[e] < INF)) vq[e] = -INF;
                 }
                 v = make_float4(vq[0], vq[1], vq[2], vq[3]);
             }
@@ -709,7 +724,7 @@ cudaError_t launch_slab_import(T* slot, unsigned long long* ups, unsigned long l
 
 template <typename T>
 size_t loop_smem_bytes() {
-    return sizeof(WarpSmem<T>) * kWarps;
+    return std::max(sizeof(WarpSmem<T>), sizeof(QueueSmem<T>)) * kWarps;
 }
 
 template <typename T>

@@ -451,10 +451,14 @@ __device__ __forceinline__ double warp_min_nn(double v) {
     return __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(mh) << 32) | ml));
 }
 template <typename T>
-__device__ __forceinline__ T warp_max(T v) {
+__device__ __forceinline__ T warp_max(T v) {            // (values >= 0)
+    if constexpr (sizeof(T) == 4) {
+        return from_bits(__reduce_max_sync(kFull, ubits(v)));
+    } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = vmax(v, __shfl_xor_sync(kFull, v, o));
-    return v;
+        for (int o = 16; o > 0; o >>= 1) v = vmax(v, __shfl_xor_sync(kFull, v, o));
+        return v;
+    }
 }
 __device__ __forceinline__ unsigned long long warp_or64(unsigned long long v) {
     const unsigned lo = __reduce_or_sync(kFull, static_cast<unsigned>(v));
@@ -496,7 +500,18 @@ struct Geo {
     int32_t GX, GY;
     int32_t goff;
     uint32_t lists;            // bit 0: keep the brick work list; bit 1: keep the group work list
+    FastDiv div_x, div_xy;     // by BX and BX*BY
 };
+
+// Coordinates of a brick (global index) in its grid.
+struct BrickAt {
+    int x, y, z;
+};
+__device__ __forceinline__ BrickAt brick_at(const Geo& G, int32_t b) {
+    const int bl = b - G.boff;
+    const int z = fast_div(bl, G.div_xy), r = bl - z * (G.BX * G.BY), y = fast_div(r, G.div_x);
+    return BrickAt{r - y * G.BX, y, z};
+}
 
 // Put brick x (global index; and, if the group work list is kept, its group)
 // on restart k+1's work lists, once per restart (the "queued" marks dedupe).
@@ -525,7 +540,7 @@ __device__ __forceinline__ void enqueue_next(const LoopParams<T>& P, const Geo& 
 // Alg. 5 for its ghost layer done first from the neighbours' copies as of the
 // end of restart k-1.
 //
-// GROUP = false: one warp, one 8^3 block.  GROUP = true: the eight warps of the
+// The eight warps of the
 // CTA march the 2x2x2 bricks of one 16^3 block together (warp w holds brick
 // (w & 1, (w >> 1) & 1, w >> 2) of the group; b < 0 for a brick outside the
 // grid, whose warp only takes part in the barriers).  The rounds then share
@@ -534,10 +549,9 @@ __device__ __forceinline__ void enqueue_next(const LoopParams<T>& P, const Geo& 
 // ghost layer on internal faces from the neighbouring warp's tile, so
 // information crosses the internal faces within the restart as it does inside
 // one block of the paper.
-template <typename T, bool GROUP>
-__device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int warp, int32_t b, unsigned gmask,
-                      int k, T bprev, T bound, bool grow, T window, int lane, MarchAcc& acc, bool publish,
-                      int32_t pf = -1) {
+template <typename T>
+__device__ void march_group(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int warp, int32_t b, unsigned gmask,
+                      int k, T bprev, T bound, bool grow, T window, int lane, MarchAcc& acc, bool publish) {
     __shared__ T s_wmin[kWarps];
     __shared__ T s_bmin[2][kWarps];            // group rounds: band minima, by round parity
     WarpSmem<T>& S = SW[warp];
@@ -571,9 +585,6 @@ __device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int
         unsigned long long wst[6];
 #pragma unroll
         for (int f = 0; f < 6; ++f) wst[f] = nbr[f] >= 0 ? __ldcg(P.stamp + nbr[f]) : kUntouched;
-        // a brick further down this restart's list (pf >= 0): its stamp now, and
-        // once it has landed (below) bulk L2 prefetches of its h/F and latest copy
-        const unsigned long long pst = (pf >= 0 && lane == 0) ? __ldcg(P.stamp + pf) : kUntouched;
         // fixed nodes (r < 0) and barrier/padding nodes (r = +inf) are never solved
         FXOB = 0;
         {
@@ -630,11 +641,6 @@ __device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int
                 else off = u;
                 load2_cg(src + off, fv0[f], fv1[f]);
             }
-        }
-        if (pf >= 0 && lane == 0) {
-            prefetch_l2(P.rr + static_cast<int64_t>(pf) * kBrick, kBrick * sizeof(T));
-            if (pst != kUntouched)
-                prefetch_l2(P.slot + (static_cast<int64_t>(pf) * 2 + stamp_copy(pst)) * kSlot, kSlot * sizeof(T));
         }
         // ---- the band at the start of the march (marked as the values land in
         // shared memory): the brick's finite nodes above the previous bound, and
@@ -696,46 +702,37 @@ __device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int
         S.fxob[lane] = 0u;
     }
     __syncwarp();
-    if constexpr (GROUP) {
-        if (FXOB & 0xFFu) atomicOr(&S.fxob[pbase >> 5], (FXOB & 0xFFu) << (pbase & 31));
-        if (FXOB >> 8) atomicOr(&S.fxob[(pbase + 64) >> 5], (FXOB >> 8) << ((pbase + 64) & 31));
-    }
+    if (FXOB & 0xFFu) atomicOr(&S.fxob[pbase >> 5], (FXOB & 0xFFu) << (pbase & 31));
+    if (FXOB >> 8) atomicOr(&S.fxob[(pbase + 64) >> 5], (FXOB >> 8) << ((pbase + 64) & 31));
 
     const T rmin_b = warp_min_nn(rlo);
     if (present) {
         acc.rmin = fminf(acc.rmin, static_cast<float>(rmin_b));
         acc.rmax = fmaxf(acc.rmax, static_cast<float>(warp_max(rhi)));
     }
-    T w;
-    if constexpr (GROUP) {
-        // one window for the group: omega times the smallest h/F of its bricks
-        if (lane == 0) s_wmin[warp] = rmin_b;
-        __syncthreads();
-        T g = s_wmin[0];
+    // one window for the group: omega times the smallest h/F of its bricks
+    if (lane == 0) s_wmin[warp] = rmin_b;
+    __syncthreads();
+    T w = s_wmin[0];
 #pragma unroll
-        for (int i = 1; i < kWarps; ++i) g = vmin(g, s_wmin[i]);
-        w = window * g;
-        __syncthreads();
-    } else {
-        w = window * rmin_b;
-    }
+    for (int i = 1; i < kWarps; ++i) w = vmin(w, s_wmin[i]);
+    w = window * w;
+    __syncthreads();
     const float tau = static_cast<float>(P.fallback_tau);
 
     // ghost layer on internal faces <- the neighbouring warps' boundary nodes
     auto refresh_internal = [&]() {
-        if constexpr (GROUP) {
 #pragma unroll
-            for (int f = 0; f < 6; ++f) {
-                if (!((gmask >> f) & 1u)) continue;
-                const WarpSmem<T>& NB = SW[warp ^ (1 << (f >> 1))];
+        for (int f = 0; f < 6; ++f) {
+            if (!((gmask >> f) & 1u)) continue;
+            const WarpSmem<T>& NB = SW[warp ^ (1 << (f >> 1))];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int uu = 2 * lane + e;
-                    S.psi[face_ghost_halo(f, uu)] = NB.psi[face_own_halo(f ^ 1, uu)];
-                }
+            for (int e = 0; e < 2; ++e) {
+                const int uu = 2 * lane + e;
+                S.psi[face_ghost_halo(f, uu)] = NB.psi[face_own_halo(f ^ 1, uu)];
             }
-            __syncwarp();
         }
+        __syncwarp();
     };
 
     // Alg. 3 for each listed node (halo index), 32 at a time; new values land
@@ -812,185 +809,98 @@ __device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int
 
     // ---- rounds of windowed ordered acceptance (Alg. 4)
     int rounds = 0;
-    if constexpr (GROUP) {
-        for (;;) {
-            T lmin = INF;
-            for (int i = lane; i < n; i += 32) lmin = vmin(lmin, vabs(S.psi[S.band[i]]));
-            T mn = warp_min_nn(lmin);
-            // (two buffers by round parity: the barriers later in the round order
-            // these reads before the writes two rounds on, so one barrier suffices)
-            T* bm = s_bmin[rounds & 1];
-            if (lane == 0) bm[warp] = mn;
-            __syncthreads();
-            T g = bm[0];
-#pragma unroll
-            for (int i = 1; i < kWarps; ++i) g = vmin(g, bm[i]);
-            mn = g;
-            if (!(mn < INF) || !(mn <= bound)) break;   // band empty, or its minimum above the bound
-            if (++rounds > kRoundCap) {
-                atomicOr(&P.ctrl->status, kStRoundCap);
-                break;
-            }
-            const T thr = vmin(mn + w, bound);
-            // accept (Remove_Min of a window), keep the rest of the band in order,
-            // and mark the accepted nodes' neighbours (Alg. 2), across internal
-            // faces in the neighbouring warp's tile
-            int kept = 0;
-            for (int base = 0; base < n; base += 32) {
-                const int i = base + lane;
-                int hh = 0;
-                bool keep = false, take = false;
-                if (i < n) {
-                    hh = S.band[i];
-                    const T v = vabs(S.psi[hh]);
-                    if (!vlt(thr, v)) {
-                        take = true;
-                        S.psi[hh] = v;
-                    } else {
-                        keep = true;
-                    }
-                }
-                const unsigned km = __ballot_sync(kFull, keep);
-                if (keep) S.band[kept + __popc(km & lt)] = static_cast<uint16_t>(hh);
-                kept += __popc(km);
-                acc.accepted += take ? 1u : 0u;
-                if (take) {
-                    const int px = hh % 10 - 1, py = (hh / 10) % 10 - 1, pz = hh / 100 - 1;
-                    auto cand = [&](int x, int yy, int z) {
-                        const bool ix = static_cast<unsigned>(x) < 8u, iy = static_cast<unsigned>(yy) < 8u,
-                                   iz = static_cast<unsigned>(z) < 8u;
-                        if (ix && iy && iz) {
-                            const int q = (z * 8 + yy) * 8 + x;
-                            atomicOr(&S.mark[q >> 5], 1u << (q & 31));
-                        } else {
-                            int f = -1;
-                            if (!ix && iy && iz) f = (x < 0) ? 0 : 1;
-                            else if (ix && !iy && iz) f = (yy < 0) ? 2 : 3;
-                            else if (ix && iy && !iz) f = (z < 0) ? 4 : 5;
-                            if (f >= 0 && ((gmask >> f) & 1u)) {
-                                const int q = (((z & 7) * 8) + (yy & 7)) * 8 + (x & 7);
-                                atomicOr(&SW[warp ^ (1 << (f >> 1))].mark[q >> 5], 1u << (q & 31));
-                            }
-                        }
-                    };
-                    cand(px - 1, py, pz);
-                    cand(px + 1, py, pz);
-                    cand(px, py - 1, pz);
-                    cand(px, py + 1, pz);
-                    cand(px, py, pz - 1);
-                    cand(px, py, pz + 1);
-                }
-            }
-            n = kept;
-            __syncthreads();
-            refresh_internal();
-            __syncthreads();
-            // candidates (brick bits, 16 per lane) -> list of halo indices; never-solved nodes dropped
-            const unsigned word = S.mark[lane >> 1] & ~S.fxob[lane >> 1];
-            const unsigned wd = (lane & 1) ? (word >> 16) : (word & 0xFFFFu);
-            __syncwarp();
-            if (lane < 16) S.mark[lane] = 0u;
-            const int total = compact(wd, 16 * lane);   // brick indices
-            for (int i = lane; i < total; i += 32) S.list[i] = static_cast<uint16_t>(halo_of(S.list[i]));
-            __syncwarp();
-            acc.solves += total;
-            solve_list(total);
-            // no barrier or refresh here: the next round's first barrier orders these
-            // writes before any other warp's marks and reads, and the ghost layer is
-            // refreshed after the next accept pass, before any solve reads it
-        }
-    } else {
-        // Halo bit vectors, one 32-bit word per lane (bit j of lane L's word is
-        // halo position 32L + j): `solv` marks the nodes that are solved (not
-        // fixed, barrier or padding); S.mark collects each round's accepted
-        // nodes, whose neighbours are the vector shifted by +-1, +-10, +-100.
-        // Every shift lands an interior node's true neighbour or a ghost
-        // position, and ghost positions are not in `solv`.
-        S.mark[lane] = 0u;
-        __syncwarp();
-        {
-            auto put = [&](int h0, unsigned bits) {
-                if (!bits) return;
-                atomicOr(&S.mark[h0 >> 5], bits << (h0 & 31));
-                if ((h0 & 31) > 24) atomicOr(&S.mark[(h0 >> 5) + 1], bits >> (32 - (h0 & 31)));
-            };
-            put(hbase, ~FXOB & 0xFFu);
-            put(hbase + 100, (~FXOB >> 8) & 0xFFu);
-        }
-        __syncwarp();
-        const unsigned solv = S.mark[lane];
-        __syncwarp();
-        S.mark[lane] = 0u;
-        __syncwarp();
+    for (;;) {
         T lmin = INF;
         for (int i = lane; i < n; i += 32) lmin = vmin(lmin, vabs(S.psi[S.band[i]]));
         T mn = warp_min_nn(lmin);
-        for (;;) {
-            if (!(mn < INF) || !(mn <= bound)) break;   // band empty, or its minimum above the bound
-            if (++rounds > kRoundCap) {
-                atomicOr(&P.ctrl->status, kStRoundCap);
-                break;
-            }
-            const T thr = vmin(mn + w, bound);
-            // accept (Remove_Min of a window) and keep the rest of the band in
-            // order, with the minimum of what is kept
-            // (the next chunk's entries are loaded before this chunk's stores, which
-            // only touch earlier band slots and the accepted nodes themselves)
-            int kept = 0;
-            T kmin = INF;
-            int hh = 0;
-            T v = INF;
-            if (lane < n) {
-                hh = S.band[lane];
-                v = vabs(S.psi[hh]);
-            }
-            for (int base = 0; base < n; base += 32) {
-                const bool valid = base + lane < n;
-                int hh2 = 0;
-                T v2 = INF;
-                if (base + 32 + lane < n) {
-                    hh2 = S.band[base + 32 + lane];
-                    v2 = vabs(S.psi[hh2]);
-                }
-                const bool take = valid && !vlt(thr, v);
-                const bool keep = valid && !take;
-                if (take) {
-                    S.psi[hh] = v;
-                    atomicOr(&S.mark[hh >> 5], 1u << (hh & 31));
-                }
-                if (keep) kmin = vmin(kmin, v);
-                const unsigned km = __ballot_sync(kFull, keep);
-                if (keep) S.band[kept + __popc(km & lt)] = static_cast<uint16_t>(hh);
-                kept += __popc(km);
-                hh = hh2;
-                v = v2;
-            }
-            if (lane == 0) acc.accepted += static_cast<unsigned>(n - kept);   // every entry is taken or kept
-            n = kept;
-            __syncwarp();
-            // neighbours of the accepted nodes (Alg. 2) that are solved
-            const unsigned W = S.mark[lane];
-            unsigned wm1 = __shfl_up_sync(kFull, W, 1), wm3 = __shfl_up_sync(kFull, W, 3);
-            unsigned wm4 = __shfl_up_sync(kFull, W, 4), wp1 = __shfl_down_sync(kFull, W, 1);
-            unsigned wp3 = __shfl_down_sync(kFull, W, 3), wp4 = __shfl_down_sync(kFull, W, 4);
-            if (lane < 1) wm1 = 0u;
-            if (lane < 3) wm3 = 0u;
-            if (lane < 4) wm4 = 0u;
-            if (lane > 30) wp1 = 0u;
-            if (lane > 28) wp3 = 0u;
-            if (lane > 27) wp4 = 0u;
-            const unsigned d = (__funnelshift_l(wm1, W, 1) | __funnelshift_l(wm1, W, 10) | __funnelshift_l(wm4, wm3, 4) |
-                                __funnelshift_r(W, wp1, 1) | __funnelshift_r(W, wp1, 10) | __funnelshift_r(wp3, wp4, 4)) &
-                               solv;
-            S.mark[lane] = 0u;
-            const int total = compact(d, 32 * lane);
-            acc.solves += total;
-            const T smin = solve_list(total);
-            mn = warp_min_nn(vmin(kmin, smin));
+        // (two buffers by round parity: the barriers later in the round order
+        // these reads before the writes two rounds on, so one barrier suffices)
+        T* bm = s_bmin[rounds & 1];
+        if (lane == 0) bm[warp] = mn;
+        __syncthreads();
+        T g = bm[0];
+#pragma unroll
+        for (int i = 1; i < kWarps; ++i) g = vmin(g, bm[i]);
+        mn = g;
+        if (!(mn < INF) || !(mn <= bound)) break;   // band empty, or its minimum above the bound
+        if (++rounds > kRoundCap) {
+            atomicOr(&P.ctrl->status, kStRoundCap);
+            break;
         }
+        const T thr = vmin(mn + w, bound);
+        // accept (Remove_Min of a window), keep the rest of the band in order,
+        // and mark the accepted nodes' neighbours (Alg. 2), across internal
+        // faces in the neighbouring warp's tile
+        int kept = 0;
+        for (int base = 0; base < n; base += 32) {
+            const int i = base + lane;
+            int hh = 0;
+            bool keep = false, take = false;
+            if (i < n) {
+                hh = S.band[i];
+                const T v = vabs(S.psi[hh]);
+                if (!vlt(thr, v)) {
+                    take = true;
+                    S.psi[hh] = v;
+                } else {
+                    keep = true;
+                }
+            }
+            const unsigned km = __ballot_sync(kFull, keep);
+            if (keep) S.band[kept + __popc(km & lt)] = static_cast<uint16_t>(hh);
+            kept += __popc(km);
+            acc.accepted += take ? 1u : 0u;
+            if (take) {
+                const int px = hh % 10 - 1, py = (hh / 10) % 10 - 1, pz = hh / 100 - 1;
+                const T va = S.psi[hh];                 // (accepted: sign clear)
+                auto cand = [&](int x, int yy, int z) {
+                    const bool ix = static_cast<unsigned>(x) < 8u, iy = static_cast<unsigned>(yy) < 8u,
+                               iz = static_cast<unsigned>(z) < 8u;
+                    if (ix && iy && iz) {
+                        const int q = (z * 8 + yy) * 8 + x;
+                        atomicOr(&S.mark[q >> 5], 1u << (q & 31));
+                    } else {
+                        int f = -1;
+                        if (!ix && iy && iz) f = (x < 0) ? 0 : 1;
+                        else if (ix && !iy && iz) f = (yy < 0) ? 2 : 3;
+                        else if (ix && iy && !iz) f = (z < 0) ? 4 : 5;
+                        if (f >= 0 && ((gmask >> f) & 1u)) {
+                            const int q = (((z & 7) * 8) + (yy & 7)) * 8 + (x & 7);
+                            atomicOr(&SW[warp ^ (1 << (f >> 1))].mark[q >> 5], 1u << (q & 31));
+                        }
+                    }
+                };
+                // only neighbours above the accepted value can be lowered by it (beyond
+                // an internal face the ghost layer's copy: never below the node itself)
+                const int pi = ((pz + 1) * 10 + (py + 1)) * 10 + px + 1;
+                if (px > -1 && vlt(va, vabs(S.psi[pi - 1]))) cand(px - 1, py, pz);
+                if (px < 8 && vlt(va, vabs(S.psi[pi + 1]))) cand(px + 1, py, pz);
+                if (py > -1 && vlt(va, vabs(S.psi[pi - 10]))) cand(px, py - 1, pz);
+                if (py < 8 && vlt(va, vabs(S.psi[pi + 10]))) cand(px, py + 1, pz);
+                if (pz > -1 && vlt(va, vabs(S.psi[pi - 100]))) cand(px, py, pz - 1);
+                if (pz < 8 && vlt(va, vabs(S.psi[pi + 100]))) cand(px, py, pz + 1);
+            }
+        }
+        n = kept;
+        __syncthreads();
+        refresh_internal();
+        __syncthreads();
+        // candidates (brick bits, 16 per lane) -> list of halo indices; never-solved nodes dropped
+        const unsigned word = S.mark[lane >> 1] & ~S.fxob[lane >> 1];
+        const unsigned wd = (lane & 1) ? (word >> 16) : (word & 0xFFFFu);
+        __syncwarp();
+        if (lane < 16) S.mark[lane] = 0u;
+        const int total = compact(wd, 16 * lane);   // brick indices
+        for (int i = lane; i < total; i += 32) S.list[i] = static_cast<uint16_t>(halo_of(S.list[i]));
+        __syncwarp();
+        acc.solves += total;
+        solve_list(total);
+        // no barrier or refresh here: the next round's first barrier orders these
+        // writes before any other warp's marks and reads, and the ghost layer is
+        // refreshed after the next accept pass, before any solve reads it
     }
     acc.rounds += rounds;
-    if constexpr (GROUP) __syncthreads();
+    __syncthreads();
     if (!present) return;
 
     // ---- Upsilon: own face nodes lowered in this march, per face (face-local bit
@@ -1014,7 +924,7 @@ __device__ void march(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
             um[f] = warp_or64(um[f]);
-            if (GROUP && ((gmask >> f) & 1u)) um[f] = 0ull;
+            if (((gmask >> f) & 1u)) um[f] = 0ull;
         }
 
         // ---- write the other copy, then publish it
@@ -1090,8 +1000,8 @@ template <typename T>
 __device__ bool wait_ready(const LoopParams<T>& P, const Geo& G, int32_t b, int k, int lane) {
     int32_t x = -1;
     if (lane < 7) {
-        const int bl = b - G.boff;
-        const int bx = bl % G.BX, by = (bl / G.BX) % G.BY, bz = bl / (G.BX * G.BY);
+        const BrickAt at = brick_at(G, b);
+        const int bx = at.x, by = at.y, bz = at.z;
         if (lane == 6) x = b;
         else if (lane == 0) x = bx > 0 ? b - 1 : -1;
         else if (lane == 1) x = bx < G.BX - 1 ? b + 1 : -1;

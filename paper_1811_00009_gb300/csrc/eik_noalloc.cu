@@ -260,6 +260,8 @@ eik_status eik_solve_noalloc(const int32_t dims[3], double h, const float* F, in
         L.BX = BX;
         L.BY = BY;
         L.BZ = BZ;
+        L.div_x = eikg::make_fastdiv(L.BX);
+        L.div_xy = eikg::make_fastdiv(static_cast<int64_t>(L.BX) * L.BY);
         L.nbricks = nb;
         L.slot = slot;
         L.ups = ups;
@@ -278,6 +280,7 @@ eik_status eik_solve_noalloc(const int32_t dims[3], double h, const float* F, in
         L.window_f = static_cast<float>(P.window);
         L.width = P.width;
         L.fallback_tau = P.fallback_tau;
+        L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.wait_limit = P.wait_polls > 0 ? P.wait_polls : eikg::kWaitPolls;
         L.sched = EIK_SCHED_FIXED;

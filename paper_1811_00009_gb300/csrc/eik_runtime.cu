@@ -626,6 +626,8 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         L.BX = c->BX;
         L.BY = c->BY;
         L.BZ = c->BZ;
+        L.div_x = eikg::make_fastdiv(L.BX);
+        L.div_xy = eikg::make_fastdiv(static_cast<int64_t>(L.BX) * L.BY);
         L.nbricks = c->nbricks;
         L.slot = static_cast<T*>(c->slot);
         L.ups = c->ups;
@@ -651,6 +653,7 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         L.window = P.window;
         L.window_f = static_cast<float>(P.window);
         L.fallback_tau = P.fallback_tau;
+        L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.width = P.width;
         L.wait_limit = P.wait_polls > 0 ? P.wait_polls : eikg::kWaitPolls;

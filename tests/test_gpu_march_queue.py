@@ -1,0 +1,64 @@
+"""The queue march of the 8^3 blocks (eik_march8.cuh) where it can go wrong: rough speeds (many stages in a
+march, corrections of accepted values), barriers, sources on block faces, grids of one node to a few blocks with
+ragged edges, and windows and strides from one node a stage to the whole block at once.
+
+Every variant must give the discrete solution of the FP64 oracle within the precision bars of the parity tests
+(FP64: relative 1e-12; FP32: 1e-5 of the largest psi, the accumulated rounding of one root per node along a
+characteristic) and must equal the first variant bit for bit (the update is monotone, so the order of the work
+does not matter).
+"""
+import math
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def eik():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1811_00009_gb300 import build
+    build.build()
+    import paper_1811_00009_gb300 as E
+    return E
+
+
+VARIANTS = [dict(stride=2.0), dict(stride=0.3), dict(stride=1.0, window=1e-3), dict(stride=5.0, window=0.5),
+            dict(stride=math.inf), dict(stride=math.inf, window=50.0), dict(stride=3.0, fallback_tau=1.0)]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (8, 8, 8), (9, 7, 8), (17, 8, 25), (31, 33, 16)])
+def test_rough_speeds_and_barriers(eik, orc, dims, precision):
+    n = int(np.prod(dims))
+    h = synth.grid_h(dims)
+    u = synth.uniform(91 + n, 2, 2 * n)
+    F = (10.0 ** (2.0 * u[:n] - 1.0)).reshape(dims[::-1])             # 0.1 .. 10
+    F[(u[n:] < 0.12).reshape(dims[::-1])] = 0.0
+    F[0, 0, 0] = 1.0
+    F = synth.round_to(F, precision)
+    src = [[0.0, 0.0, 0.0]]
+    if min(dims) > 8:
+        src += [[8 * h, 8 * h, 7.5 * h], [(dims[0] - 1) * h, 0.3 * h, 9 * h]]
+    ref = orc.fmm(F, h, src)
+    fin = np.isfinite(ref)
+    dt = np.float32 if precision == "fp32" else np.float64
+    base = None
+    with eik.Solver(dims, h, np.ascontiguousarray(F.astype(dt)), precision) as S:
+        S.add_sources(src)
+        for v in VARIANTS:
+            kw = dict(v)
+            S.solve(kw.pop("stride") * h, block_dim=8, **kw)
+            psi = S.result()
+            assert np.array_equal(np.isfinite(psi), fin), v
+            if precision == "fp64":
+                assert np.all(np.abs(psi[fin] - ref[fin]) <= 1e-12 * ref[fin]), v
+            else:
+                assert np.max(np.abs(psi[fin].astype(np.float64) - ref[fin])) <= 1e-5 * ref[fin].max(), v
+            base = psi.copy() if base is None else base
+            assert np.array_equal(psi, base), v
