@@ -99,19 +99,44 @@ __device__ __forceinline__ void batch_bounds_ahead(const LoopParams<T>& P, int k
     __threadfence();
 }
 
+// The restart the control block describes -> the CTA's state (one lane).
+template <typename T>
+__device__ void load_batch_restart(const LoopParams<T>& P, CtaLoop& S) {
+    const Ctrl* C = P.ctrl;
+    const int k = __ldcg(&C->k), done = __ldcg(&C->done);
+    const unsigned gen = __ldcg(&C->bar_gen);
+    const int n = __ldcg(&C->count[k % kRing]), used = __ldcg(&C->used[(k + kRing - 1) % kRing]);
+    S.k = k;
+    S.done = done;
+    S.n = n;
+    S.used = P.early ? used : 0;
+    S.gen = gen;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_loop(LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
-    __shared__ LoopState s_state[kWarps];
+    __shared__ CtaLoop S;
     __shared__ MarchAcc s_acc[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
     QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
-    LoopState& L = s_state[warp];              // the loop's bookkeeping, kept out of registers
     Ctrl* C = P.ctrl;
-    if (threadIdx.x == 0) s_arrived = 0;
+    MarchAcc& A = s_acc[warp];
+    if (threadIdx.x == 0) {
+        s_arrived = 0;
+        S.arrived = 0;
+        S.stop = 0;
+        S.token = 0;
+        S.claim = 0ull;
+        S.drained = -1;
+        reset_acc(S.acc);
+        load_batch_restart(P, S);
+        S.rel = S.gen;
+    }
+    if (lane == 0) reset_acc(A);
     init_queue_smem(SQ[warp], lane);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -119,150 +144,102 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_l
         C->t_begin = t0;
         C->t_restart = t0;
     }
-    if (lane == 0) L.claim = -1;
-    MarchAcc& A = s_acc[warp];
-    if (lane == 0) reset_acc(A);
     bool any = false;
     for (;;) {
-        const int k = __ldcg(&C->k);
+        const int k = S.k;
         const int s = k % kRing;
-        const bool early_k = P.early != 0;
-        if (P.early) clear_used_slot(P, k);
-        // ---- 16^3 blocks: one CTA per group of 2x2x2 bricks (the CTA goes on only as a whole)
-        if (!cta_go(C, true, lane, &s_arrived)) return;
-        {
-            const int n = __ldcg(&C->gcount[s]);
-            MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
-            bool grouped = false;
-            for (;;) {
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    const int i = atomicAdd(&C->ghead[s], 1);
-                    s_item = -1;
-                    if (i < n) s_item = __ldcg(P.glist[s] + i);
+        const unsigned gen = S.gen;
+        clear_used_slot(P, k, S.used);
+        // ---- 16^3 blocks (if any grid has them): one CTA per group of 2x2x2 bricks
+        // (the CTA goes on only as a whole)
+        if (P.groups) {
+            if (!cta_go(C, true, lane, &s_arrived)) return;
+            {
+                const int n = __ldcg(&C->gcount[s]);
+                MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+                bool grouped = false;
+                for (;;) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        const int i = atomicAdd(&C->ghead[s], 1);
+                        s_item = -1;
+                        if (i < n) s_item = __ldcg(P.glist[s] + i);
+                    }
+                    __syncthreads();
+                    const int g = s_item;
+                    if (g < 0) break;
+                    const int sv = __ldg(P.gsolve + g);
+                    const SolveDesc D = P.solves[sv];
+                    const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 2u, D.div_x, D.div_xy};
+                    const int gl = g - D.goff;
+                    const int gx = gl % D.GX, gy = (gl / D.GX) % D.GY, gz = gl / (D.GX * D.GY);
+                    const int bx = 2 * gx + (warp & 1), by = 2 * gy + ((warp >> 1) & 1), bz = 2 * gz + (warp >> 2);
+                    const bool in = bx < D.BX && by < D.BY && bz < D.BZ;
+                    const int32_t b = in ? D.boff + (bz * D.BY + by) * D.BX + bx : -1;
+                    unsigned gmask = 0;
+                    if (in) {
+                        if (warp & 1) gmask |= 1u;
+                        else if (bx + 1 < D.BX) gmask |= 2u;
+                        if (warp & 2) gmask |= 4u;
+                        else if (by + 1 < D.BY) gmask |= 8u;
+                        if (warp & 4) gmask |= 16u;
+                        else if (bz + 1 < D.BZ) gmask |= 32u;
+                    }
+                    march_group<T>(P, G, SW, warp, b, gmask, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
+                                   pick<T>(P.window, P.window_f), lane, acc, P.early != 0);
+                    if (threadIdx.x == 0) atomicMax(P.last_k + sv, k);
+                    grouped = true;
                 }
-                __syncthreads();
-                const int g = s_item;
-                if (g < 0) break;
-                const int sv = __ldg(P.gsolve + g);
-                const SolveDesc D = P.solves[sv];
-                const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 2u, D.div_x, D.div_xy};
-                const int gl = g - D.goff;
-                const int gx = gl % D.GX, gy = (gl / D.GX) % D.GY, gz = gl / (D.GX * D.GY);
-                const int bx = 2 * gx + (warp & 1), by = 2 * gy + ((warp >> 1) & 1), bz = 2 * gz + (warp >> 2);
-                const bool in = bx < D.BX && by < D.BY && bz < D.BZ;
-                const int32_t b = in ? D.boff + (bz * D.BY + by) * D.BX + bx : -1;
-                unsigned gmask = 0;
-                if (in) {
-                    if (warp & 1) gmask |= 1u;
-                    else if (bx + 1 < D.BX) gmask |= 2u;
-                    if (warp & 2) gmask |= 4u;
-                    else if (by + 1 < D.BY) gmask |= 8u;
-                    if (warp & 4) gmask |= 16u;
-                    else if (bz + 1 < D.BZ) gmask |= 32u;
+                if (grouped) {
+                    flush_acc(C, acc, lane);
+                    init_queue_smem(SQ[warp], lane);              // (the groups' tiles overlay it)
                 }
-                march_group<T>(P, G, SW, warp, b, gmask, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
-                               pick<T>(P.window, P.window_f), lane, acc, early_k);
-                if (threadIdx.x == 0) atomicMax(P.last_k + sv, k);
-                grouped = true;
-            }
-            if (grouped) {
-                flush_acc(C, acc, lane);
-                init_queue_smem(SQ[warp], lane);              // (the groups' tiles overlay it)
             }
         }
         // ---- 8^3 blocks, one warp per brick: this restart's list, then -- once
         // arrived at the barrier -- restart k+1's bricks whose neighbourhood has
         // finished restart k.  One march call site for both.
-        if (lane == 0) {
-            L.n = __ldcg(&C->count[s]);
-            L.waiting = 0;
-            L.polls = 0;
-            L.nap = 256;
-        }
-        __syncwarp();
+        bool waiting = false, first = true;
         for (;;) {
             int32_t b = -1;
             int kk = k;
-            if (!L.waiting) {
-                int i = -1;
-                if (lane == 0) {
-                    const int n = L.n;
-                    if (L.claim >= 0 && L.claim < n) i = L.claim;    // claimed before the entry existed
-                    else {
-                        const int j = atomicAdd(&C->head[s], 1);
-                        if (j < n) i = j;
-                    }
-                    L.claim = -1;
-                }
-                i = __shfl_sync(kFull, i, 0);
-                if (i >= 0) b = take_entry(P.list[s], i, false, 0, lane);
-                if (b < 0) {
-                    if (any) flush_acc8(C, A, lane);
+            if (!waiting) {
+                const int i = S.n > 0 ? next_entry(C, S, k, s, first, lane) : -1;
+                first = false;
+                if (i >= 0) {
+                    b = __ldcg(P.list[s] + i);
+                } else {
+                    const bool last = barrier_arrive(C, S, A, any, lane);
                     any = false;
-                    unsigned gen;
-                    if (barrier_arrive(C, lane, &gen)) {
+                    if (last) {
                         batch_bounds_ahead(P, k, lane);
                         if (lane == 0) batch_restart_end<T>(P);
                         barrier_release(C, lane, gen);
-                        break;
                     }
-                    if (lane == 0) {
-                        L.gen = gen;
-                        L.waiting = 1;
-                    }
-                    __syncwarp();
+                    waiting = true;
                     continue;
                 }
             } else {
-                const int st = barrier_poll(C, lane, L.gen);
+                const int st = wait_or_work(P, S, k, gen, P.early != 0, lane, &b, [&]() { load_batch_restart(P, S); });
                 if (st == 2) return;
                 if (st == 1) break;
-                if (early_k) {
-                    int claim = L.claim;
-                    b = early_entry(C, P.list[(k + 1) % kRing], (k + 1) % kRing, claim, P.wait_limit, lane);
-                    if (lane == 0) L.claim = claim;
-                }
-                if (b >= 0) {
-                    const SolveDesc D = P.solves[__ldg(P.bsolve + b)];
-                    const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u, D.div_x, D.div_xy};
-                    if (!wait_ready(P, G, b, k, lane)) b = -2;
-                }
-                if (b == -2) {
-                    give_up(C, lane);
-                    return;
-                }
-                if (b < 0) {
-                    int quit = 0;
-                    unsigned nap = 0;
-                    if (lane == 0) {
-                        quit = ++L.polls > P.wait_limit;
-                        nap = L.nap;
-                        if (L.nap < 4096) L.nap <<= 1;
-                    }
-                    if (__shfl_sync(kFull, quit, 0)) {
-                        give_up(C, lane);
-                        return;
-                    }
-                    __nanosleep(__shfl_sync(kFull, nap, 0));
-                    continue;
-                }
                 kk = k + 1;
-                if (lane == 0) {
-                    L.polls = 0;
-                    L.nap = 256;
-                }
             }
-            __syncwarp();
             const int sv = __ldg(P.bsolve + b);
             const SolveDesc D = P.solves[sv];
             const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 1u, D.div_x, D.div_xy};
+            if (kk > k && !wait_ready(P, G, b, k, lane)) {
+                if (lane == 0) vol_set(S.stop, 1);
+                give_up(C, lane);
+                return;
+            }
             march8<T>(P, G, SQ[warp], A, b, kk, batch_bound(P, sv, kk - 1), batch_bound(P, sv, kk), true,
-                            pick<T>(P.window, P.window_f), lane, early_k || kk > k);
+                      pick<T>(P.window, P.window_f), lane, P.early != 0);
             if (lane == 0) atomicMax(P.last_k + sv, kk);
             any = true;
         }
-        if (__ldcg(&C->done)) return;
+        __syncwarp();
+        if (S.done) return;
     }
 }
 
@@ -663,6 +640,7 @@ eik_status batch_queue(eik_batch* b, const std::vector<eik_batch_tile>& tiles, i
         L.nbricks = b->nbricks;
         L.ngroups = b->ngroups;
         L.early = 1;
+        L.groups = genq.empty() ? 0 : 1;
         L.rr = static_cast<const T*>(b->rr);
         for (int r = 0; r < eikg::kRing; ++r) {
             L.list[r] = b->lists + r * b->nbricks;

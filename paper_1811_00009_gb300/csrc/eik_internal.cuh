@@ -60,11 +60,15 @@ constexpr int kStRestartCap = 2;   // max_restarts reached with work left
 constexpr int kStRoundCap = 4;     // a march exceeded its round cap
 
 // Control block of one restart loop, in device memory.  Written by the CTA
-// that arrives last at each grid barrier, read by all after the release.
+// that arrives last at each grid barrier, read by all after the release (one
+// warp of each CTA reads it for the CTA).
 struct Ctrl {
-    unsigned int bar_count;
-    unsigned int bar_gen;
-    int32_t pad_bar[30];       // the barrier words in a cache line of their own (polled by waiting warps)
+    unsigned int bar_count;    // CTAs that have arrived at the restart barrier
+    unsigned int bar_gen;      // restart barriers passed
+    int32_t pad_bar[30];       // the barrier words in a cache line of their own (polled by waiting CTAs)
+    unsigned int sync_count;   // the barrier inside a restart (grid_sync)
+    unsigned int sync_gen;
+    int32_t pad_sync[30];
     int32_t k;                 // current restart (1-based)
     int32_t done;
     int32_t status;
@@ -86,7 +90,8 @@ struct Ctrl {
     unsigned long long t_restart;
     unsigned long long t_end;
     // accumulators of the current restart
-    unsigned long long r_accepted, r_band, r_solves, r_updates, r_fallbacks, r_rounds;
+    // (in the order of MarchAcc's fields: a warp's lanes add them in parallel)
+    unsigned long long r_accepted, r_band, r_fallbacks, r_updates, r_solves, r_rounds;
     unsigned int r_rmin_bits, r_rmax_bits;
     // totals
     unsigned long long marches, accepted, solves, updates, fallbacks, rounds;

@@ -214,7 +214,7 @@ __device__ void restart_end(const LoopParams<T>& P, int lane, float* scratch) {
 // the launch, then a grid barrier; false if a wait ran out.  Out of line: it
 // runs only at 16^3 restarts of a learned or random schedule.
 __device__ __noinline__ bool groups_from_bricks(Ctrl* C, const int32_t* list, int32_t* qgroup, int32_t* glist, int s,
-                                                int k, int BX, int BY, int GX, int GY, int lane, long long limit) {
+                                                int k, int BX, int BY, int GX, int GY, long long limit) {
     const int nb = __ldcg(&C->count[s]);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
         const int32_t x = __ldcg(list + i);
@@ -225,8 +225,35 @@ __device__ __noinline__ bool groups_from_bricks(Ctrl* C, const int32_t* list, in
             glist[pos] = g;
         }
     }
-    __threadfence();
-    return grid_sync(C, lane, limit);
+    return grid_sync(C, limit);
+}
+
+// The restart the control block describes -> the CTA's state (one lane).
+template <typename T>
+__device__ void load_restart(const LoopParams<T>& P, CtaLoop& S) {
+    const Ctrl* C = P.ctrl;
+    const int k = __ldcg(&C->k), done = __ldcg(&C->done), mode = __ldcg(&C->mode);
+    const unsigned gen = __ldcg(&C->bar_gen);
+    const double bound = __ldcg(&C->bound), bprev = __ldcg(&C->bound_prev);
+    const int n = __ldcg(&C->count[k % kRing]), used = __ldcg(&C->used[(k + kRing - 1) % kRing]);
+    double ns;
+    int nm;
+    next_restart_of(P, C, &ns, &nm);
+    S.k = k;
+    S.done = done;
+    S.mode = mode;
+    S.n = mode == 8 ? n : 0;
+    S.used = P.early ? used : 0;
+    S.gen = gen;
+    S.early = (P.early && mode == 8 && nm == 8) ? 1 : 0;
+    S.bound = bound;
+    S.bprev = bprev;
+    S.next_bound = fmin(bound + ns, P.width);           // restart k+1's bound
+    S.bound_f = __double2float_rd(bound);
+    S.bprev_f = __double2float_rd(bprev);
+    S.next_f = __double2float_rd(S.next_bound);
+    S.grow = bound < P.width;
+    S.grow_next = S.next_bound < P.width;
 }
 
 template <typename T>
@@ -234,14 +261,27 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
-    __shared__ LoopState s_state[kWarps];
+    __shared__ CtaLoop S;
     __shared__ MarchAcc s_acc[kWarps];
+    __shared__ WarpLoop s_warp[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
     QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
-    LoopState& L = s_state[warp];              // the loop's bookkeeping, kept out of registers
     Ctrl* C = P.ctrl;
-    if (threadIdx.x == 0) s_arrived = 0;
+    MarchAcc& A = s_acc[warp];
+    WarpLoop& L = s_warp[warp];
+    if (threadIdx.x == 0) {
+        s_arrived = 0;
+        S.arrived = 0;
+        S.stop = 0;
+        S.token = 0;
+        S.claim = 0ull;
+        S.drained = -1;
+        reset_acc(S.acc);
+        load_restart(P, S);
+        S.rel = S.gen;
+    }
+    if (lane == 0) reset_acc(A);
     init_queue_smem(SQ[warp], lane);
     __syncthreads();
     // Work lists the marches fill: the brick list, and for fixed 16^3 blocks
@@ -255,38 +295,17 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
         C->t_begin = t0;
         C->t_restart = t0;
     }
-    if (lane == 0) L.claim = -1;
-    MarchAcc& A = s_acc[warp];
-    if (lane == 0) reset_acc(A);
-    bool any = false;                          // acc holds something to flush
+    bool any = false;                          // A holds something to flush
     for (;;) {
-        const int k = __ldcg(&C->k);
-        const int mode = __ldcg(&C->mode);
+        const int k = S.k;
         const int s = k % kRing;
-        if (P.early) clear_used_slot(P, k);
-        if (lane == 0) {
-            L.bound = __ldcg(&C->bound);
-            L.bprev = __ldcg(&C->bound_prev);
-            double ns;
-            int nm;
-            next_restart_of(P, C, &ns, &nm);
-            L.next_bound = fmin(L.bound + ns, P.width);         // restart k+1's bound
-            L.bound_f = __double2float_rd(L.bound);
-            L.bprev_f = __double2float_rd(L.bprev);
-            L.next_f = __double2float_rd(L.next_bound);
-            L.grow = L.bound < P.width;
-            L.grow_next = L.next_bound < P.width;
-            L.early = (P.early && mode == 8 && nm == 8) ? 1 : 0;
-            L.n = (mode == 8) ? __ldcg(&C->count[s]) : 0;
-            L.waiting = 0;
-            L.polls = 0;
-            L.nap = 256;
-        }
-        __syncwarp();
-        if (mode == 16) {
+        const unsigned gen = S.gen;
+        keep_restart(L, S, lane);
+        clear_used_slot(P, k, S.used);
+        if (S.mode == 16) {
             const bool ok = (G.lists & 2u) ||
                             groups_from_bricks(C, P.list[s], P.qgroup + static_cast<int64_t>(s) * P.ngroups,
-                                               P.glist[s], s, k, P.BX, P.BY, P.GX, P.GY, lane, P.wait_limit);
+                                               P.glist[s], s, k, P.BX, P.BY, P.GX, P.GY, P.wait_limit);
             if (!cta_go(C, ok, lane, &s_arrived)) return;
             // one CTA per group of 2x2x2 bricks
             MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
@@ -315,8 +334,8 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
                     if (warp & 4) gmask |= 16u;
                     else if (bz + 1 < P.BZ) gmask |= 32u;
                 }
-                march_group<T>(P, G, SW, warp, b, gmask, k, pick<T>(L.bprev, L.bprev_f), pick<T>(L.bound, L.bound_f),
-                               L.grow != 0, pick<T>(P.window, P.window_f), lane, acc, L.early != 0);
+                march_group<T>(P, G, SW, warp, b, gmask, k, pick<T>(S.bprev, S.bprev_f), pick<T>(S.bound, S.bound_f),
+                               S.grow != 0, pick<T>(P.window, P.window_f), lane, acc, S.early != 0);
                 grouped = true;
             }
             if (grouped) flush_acc(C, acc, lane);
@@ -324,92 +343,52 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
         }
         // One warp per 8^3 brick: this restart's list, then -- once arrived at
         // the barrier -- restart k+1's bricks whose neighbourhood has finished
-        // restart k (fixed stride and 8^3 blocks only; the next bound is then
-        // known).  One march call site for both.
+        // restart k (8^3 blocks only; the next bound is then known).  One march
+        // call site for both.
+        bool waiting = false, first = true;
         for (;;) {
             int32_t b = -1, pf = -1;
             int kk = k;
-            if (!L.waiting) {
-                int i = -1;
-                if (lane == 0) {
-                    const int n = L.n;
-                    if (L.claim >= 0 && L.claim < n) i = L.claim;    // claimed before the entry existed
-                    else {
-                        const int j = atomicAdd(&C->head[s], 1);
-                        if (j < n) i = j;
-                    }
-                    L.claim = -1;
-                }
-                i = __shfl_sync(kFull, i, 0);
+            if (!waiting) {
+                const int i = S.n > 0 ? next_entry(C, S, k, s, first, lane) : -1;
+                first = false;
                 if (i >= 0) {
-                    b = take_entry(P.list[s], i, false, 0, lane);
+                    b = __ldcg(P.list[s] + i);
                     // the entry one launch-width further down, for the march to prefetch
                     const int i2 = i + static_cast<int>(gridDim.x) * kWarps;
-                    if (i2 < L.n) pf = __ldcg(P.list[s] + i2);
+                    if (i2 < S.n) pf = __ldcg(P.list[s] + i2);
                     if (pf >= P.nbricks) pf = -1;
-                }
-                if (b < 0) {
-                    if (any) flush_acc8(C, A, lane);
+                } else {
+                    const bool last = barrier_arrive(C, S, A, any, lane);
                     any = false;
-                    unsigned gen;
-                    if (barrier_arrive(C, lane, &gen)) {
+                    if (last) {
                         restart_end<T>(P, lane, reinterpret_cast<float*>(SQ + warp));
                         init_queue_smem(SQ[warp], lane);      // (the weights were staged there)
                         barrier_release(C, lane, gen);
-                        break;
                     }
-                    if (lane == 0) {
-                        L.gen = gen;
-                        L.waiting = 1;
-                    }
-                    __syncwarp();
+                    waiting = true;
                     continue;
                 }
             } else {
-                const int st = barrier_poll(C, lane, L.gen);
+                const int st = wait_or_work(P, S, k, gen, L.early != 0, lane, &b, [&]() { load_restart(P, S); });
                 if (st == 2) return;
                 if (st == 1) break;
-                if (L.early) {
-                    int claim = L.claim;
-                    b = early_entry(C, P.list[(k + 1) % kRing], (k + 1) % kRing, claim, P.wait_limit, lane);
-                    if (lane == 0) L.claim = claim;
-                }
-                if (b >= 0 && !wait_ready(P, G, b, k, lane)) b = -2;
-                if (b == -2) {
+                if (!wait_ready(P, G, b, k, lane)) {
+                    if (lane == 0) vol_set(S.stop, 1);
                     give_up(C, lane);
                     return;
                 }
-                if (b < 0) {
-                    int quit = 0;
-                    unsigned nap = 0;
-                    if (lane == 0) {
-                        quit = ++L.polls > P.wait_limit;
-                        nap = L.nap;
-                        if (L.nap < 4096) L.nap <<= 1;
-                    }
-                    if (__shfl_sync(kFull, quit, 0)) {
-                        give_up(C, lane);
-                        return;
-                    }
-                    __nanosleep(__shfl_sync(kFull, nap, 0));
-                    continue;
-                }
                 kk = k + 1;
-                if (lane == 0) {
-                    L.polls = 0;
-                    L.nap = 256;
-                }
             }
-            __syncwarp();
             const bool ahead = kk > k;
-            march8<T>(P, G, SQ[warp], A, b, kk,
-                            ahead ? pick<T>(L.bound, L.bound_f) : pick<T>(L.bprev, L.bprev_f),
-                            ahead ? pick<T>(L.next_bound, L.next_f) : pick<T>(L.bound, L.bound_f),
-                            (ahead ? L.grow_next : L.grow) != 0, pick<T>(P.window, P.window_f), lane,
-                            L.early != 0 || ahead, pf);
+            march8<T>(P, G, SQ[warp], A, b, kk, ahead ? pick<T>(L.bound, L.bound_f) : pick<T>(L.bprev, L.bprev_f),
+                      ahead ? pick<T>(L.next_bound, L.next_f) : pick<T>(L.bound, L.bound_f),
+                      (ahead ? L.grow_next : L.grow) != 0, pick<T>(P.window, P.window_f), lane,
+                      L.early != 0 || ahead, pf);
             any = true;
         }
-        if (__ldcg(&C->done)) return;
+        __syncwarp();
+        if (S.done) return;
     }
 }
 

@@ -961,35 +961,15 @@ __device__ void march_group(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* S
     }
 }
 
-// Work-list entry i of ring slot s.  An early taker may get an index whose
-// entry is not written yet (the enqueuer bumps the count, then stores): it
-// waits for it (bounded; -1 on timeout).  Unwritten entries are -1: a slot is
-// cleared at the start of the restart after the one that used it
-// (clear_used_slot), before it is used again two restarts later.
-__device__ __forceinline__ int32_t take_entry(const int32_t* list, int i, bool wait, long long limit, int lane) {
-    if (!wait) return __ldcg(list + i);
-    int32_t v = -1;
-    if (lane == 0) {
-        v = ld_acquire(list + i);
-        for (long long it = 0; v < 0 && it < limit; ++it) {
-            __nanosleep(32);
-            v = ld_acquire(list + i);
-        }
-    }
-    return __shfl_sync(0xffffffffu, v, 0);
-}
-
 // At the start of restart k: every thread of the launch clears its share of the
-// brick list restart k-1 used (ring slot (k-1) mod kRing), coalesced.  The
-// slot is next written in restart k+1 (by early marches of restart k+2 while
-// waiting at its barrier) at the earliest, after every warp has arrived at the
-// barrier of restart k and so has finished its share.
+// brick list restart k-1 used (ring slot (k-1) mod kRing, `used` entries),
+// coalesced.  The slot is next written in restart k+1 (by early marches of
+// restart k+2 while waiting at its barrier) at the earliest, after every warp has
+// arrived at the barrier of restart k and so has finished its share.
 template <typename T>
-__device__ __forceinline__ void clear_used_slot(const LoopParams<T>& P, int k) {
-    const int sp = (k + kRing - 1) % kRing;
-    const int m = __ldcg(&P.ctrl->used[sp]);
-    int32_t* list = P.list[sp];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) list[i] = -1;
+__device__ __forceinline__ void clear_used_slot(const LoopParams<T>& P, int k, int used) {
+    int32_t* list = P.list[(k + kRing - 1) % kRing];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < used; i += gridDim.x * blockDim.x) list[i] = -1;
 }
 
 // Before an early march of brick b at restart k+1: wait until b and each of its
@@ -1023,7 +1003,7 @@ __device__ bool wait_ready(const LoopParams<T>& P, const Geo& G, int32_t b, int 
     return true;
 }
 
-// This warp's statistics of the restart -> the control block.
+// This warp's statistics of the restart, kept in registers -> the control block.
 __device__ __forceinline__ void flush_acc(Ctrl* C, MarchAcc& acc, int lane) {
     const unsigned acc_a = __reduce_add_sync(0xffffffffu, acc.accepted);
     const unsigned acc_b = __reduce_add_sync(0xffffffffu, acc.band);
@@ -1042,37 +1022,110 @@ __device__ __forceinline__ void flush_acc(Ctrl* C, MarchAcc& acc, int lane) {
     acc = MarchAcc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
 }
 
-// Per-warp state of the restart loop, in shared memory (lane 0 writes it):
-// the march needs every register it can get.
-struct LoopState {
+// State of the restart loop shared by a CTA's warps.  The control block sits in
+// a few cache lines of one L2 slice, which serves about one access a clock: with
+// every warp of a full launch (3648) reading, polling and adding there on its own,
+// each restart spent 10-15 us in those queues (64^3 in 8^3 blocks: 36 us a restart
+// with 3648 warps, 25 us with 608).  So one warp per CTA reads it for the others,
+// polls the barrier and claims early work, and the CTA arrives once and adds its
+// statistics once.
+struct CtaLoop {
+    // the restart the CTA is in, as its poller read it
+    int k;
+    int done;
+    int mode;                  // block edge
+    int n;                     // length of the brick list
+    int used;                  // length of the list to clear
+    int early;                 // early work allowed while waiting at this restart's barrier
+    int grow, grow_next;       // bound, next_bound below width_band (pending nodes re-activate the block)
     double bound, bprev, next_bound;
     float bound_f, bprev_f, next_f;    // the same rounded down to single precision
-    int grow, grow_next;       // bound, next_bound below width_band (pending nodes re-activate the block)
-    int n;                     // length of this restart's brick list
-    int early;                 // early work allowed while waiting at this restart's barrier
-    int waiting;               // arrived at the barrier
-    unsigned gen;              // barrier generation to wait past
-    int polls;
-    unsigned nap;
-    int claim;                 // entry of the next restart's list claimed while waiting (-1: none)
+    unsigned gen;              // barrier generation while in this restart
+    // its barrier
+    unsigned rel;              // generation last seen by the CTA
+    unsigned arrived;          // warps that have arrived
+    int stop;                  // a wait ran out: leave
+    int token;                 // 1: a warp polls for the CTA
+    unsigned long long claim;  // entry of a coming restart's list claimed while waiting: restart << 32 | index
+    int drained;               // restart whose list a warp found handed out
+    MarchAcc acc;              // the CTA's statistics of the restart
 };
 
-// Grid barrier at the end of a restart, one warp at a time: every warp of the
-// launch arrives on its own (lane 0's atomic), and the warp arriving last does
-// the restart bookkeeping and then releases the others by bumping bar_gen.
-// barrier_arrive returns true for that last warp; *gen gets the generation the
-// others wait to see change.
-__device__ __forceinline__ bool barrier_arrive(Ctrl* C, int lane, unsigned* gen) {
-    unsigned g = 0;
+// What a warp keeps of its restart once it has arrived at the barrier (the CTA's
+// state may then become the next restart's), in shared memory: a march needs its
+// registers.
+struct WarpLoop {
+    double bound, bprev, next_bound;
+    float bound_f, bprev_f, next_f;
+    int grow, grow_next, early;
+};
+__device__ __forceinline__ void keep_restart(WarpLoop& L, const CtaLoop& S, int lane) {
+    if (lane == 0) {
+        L.bound = S.bound;
+        L.bprev = S.bprev;
+        L.next_bound = S.next_bound;
+        L.bound_f = S.bound_f;
+        L.bprev_f = S.bprev_f;
+        L.next_f = S.next_f;
+        L.grow = S.grow;
+        L.grow_next = S.grow_next;
+        L.early = S.early;
+    }
+    __syncwarp();
+}
+
+template <typename V>
+__device__ __forceinline__ V vol(const V& x) {
+    return *const_cast<const volatile V*>(&x);
+}
+template <typename V>
+__device__ __forceinline__ void vol_set(V& x, V v) {
+    *const_cast<volatile V*>(&x) = v;
+}
+
+__device__ __forceinline__ void reset_acc(MarchAcc& A) {
+    A = MarchAcc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
+}
+
+// One warp arrives at the restart barrier: its statistics (A, if any) go to the
+// CTA's; the CTA's last warp adds those to the control block and arrives for the
+// CTA.  True for the launch's last arrival, which then runs the restart's
+// bookkeeping and releases the others.
+__device__ __forceinline__ bool barrier_arrive(Ctrl* C, CtaLoop& S, MarchAcc& A, bool any, int lane) {
+    if (any) {
+        unsigned* from = reinterpret_cast<unsigned*>(&A);
+        unsigned* to = reinterpret_cast<unsigned*>(&S.acc);
+        if (lane < 6) atomicAdd(to + lane, from[lane]);
+        if (lane == 6) atomicMin(to + 6, from[6]);       // (bits of values >= 0)
+        if (lane == 7) atomicMax(to + 7, from[7]);
+        __syncwarp();
+        if (lane == 0) reset_acc(A);
+    }
+    __syncwarp();
     int last = 0;
     if (lane == 0) {
-        g = ld_acquire(&C->bar_gen);
         __threadfence();
-        last = atomicAdd(&C->bar_count, 1u) == gridDim.x * (blockDim.x >> 5) - 1;
+        last = atomicAdd(&S.arrived, 1u) == (blockDim.x >> 5) - 1;
         if (last) __threadfence();
     }
-    *gen = __shfl_sync(0xffffffffu, g, 0);
-    return __shfl_sync(0xffffffffu, last, 0) != 0;
+    if (!__shfl_sync(kFull, last, 0)) return false;
+    {
+        const unsigned v = lane < 8 ? reinterpret_cast<unsigned*>(&S.acc)[lane] : 0u;
+        if (lane < 6 && v != 0u) atomicAdd(&C->r_accepted + lane, static_cast<unsigned long long>(v));
+        if (lane == 6) atomicMin(&C->r_rmin_bits, v);
+        if (lane == 7) atomicMax(&C->r_rmax_bits, v);
+        __syncwarp();
+        if (lane == 0) reset_acc(S.acc);
+    }
+    __syncwarp();
+    last = 0;
+    if (lane == 0) {
+        S.arrived = 0u;                       // (no warp arrives again before this barrier is passed)
+        __threadfence();
+        last = atomicAdd(&C->bar_count, 1u) == gridDim.x - 1;
+        if (last) __threadfence();
+    }
+    return __shfl_sync(kFull, last, 0) != 0;
 }
 __device__ __forceinline__ void barrier_release(Ctrl* C, int lane, unsigned gen) {
     __syncwarp();
@@ -1081,15 +1134,6 @@ __device__ __forceinline__ void barrier_release(Ctrl* C, int lane, unsigned gen)
         __threadfence();
         st_release(&C->bar_gen, gen + 1);
     }
-}
-// 1: released; 2: a wait somewhere ran out (kStWaitTimeout); 0: keep waiting.
-__device__ __forceinline__ int barrier_poll(Ctrl* C, int lane, unsigned gen) {
-    int state = 0;
-    if (lane == 0) {
-        if (ld_acquire(&C->bar_gen) != gen) state = 1;
-        else if (__ldcg(&C->status) & kStWaitTimeout) state = 2;
-    }
-    return __shfl_sync(0xffffffffu, state, 0);
 }
 
 // A warp that gives up on a wait: the status bit, made visible to every other
@@ -1120,45 +1164,139 @@ __device__ __forceinline__ bool cta_go(const Ctrl* C, bool ok, int lane, int* s_
     return stop == 0 && all;
 }
 
-// A grid barrier inside a restart (no bookkeeping): every warp of the launch
-// arrives; false if this or another wait ran out (the status then says so).
-__device__ inline bool grid_sync(Ctrl* C, int lane, long long limit) {
-    unsigned gen;
-    if (barrier_arrive(C, lane, &gen)) {
-        barrier_release(C, lane, gen);
-        return true;
-    }
-    unsigned nap = 32;
-    for (long long it = 0;; ++it) {
-        const int st = barrier_poll(C, lane, gen);
-        if (st == 1) return true;
-        if (st == 2) return false;
-        if (it > limit) {
-            give_up(C, lane);
-            return false;
+// A grid barrier inside a restart (no bookkeeping), by every warp of the launch:
+// the CTA's first thread arrives and waits for all.  False if this or another
+// wait ran out, or the first warp has left.
+__device__ inline bool grid_sync(Ctrl* C, long long limit) {
+    __threadfence();
+    __syncthreads();
+    int ok = 0;
+    if (threadIdx.x == 0) {
+        const unsigned gen = ld_acquire(&C->sync_gen);
+        __threadfence();
+        if (atomicAdd(&C->sync_count, 1u) == gridDim.x - 1) {
+            C->sync_count = 0;
+            __threadfence();
+            st_release(&C->sync_gen, gen + 1);
+            ok = 1;
+        } else {
+            unsigned nap = 32;
+            for (long long it = 0;; ++it) {
+                if (ld_acquire(&C->sync_gen) != gen) {
+                    ok = 1;
+                    break;
+                }
+                if (__ldcg(&C->status) & kStWaitTimeout) break;
+                if (it > limit) {
+                    atomicOr(&C->status, kStWaitTimeout);
+                    __threadfence();
+                    break;
+                }
+                __nanosleep(nap);
+                if (nap < 1024) nap <<= 1;
+            }
         }
-        __nanosleep(nap);
-        if (nap < 1024) nap <<= 1;
     }
+    return __syncthreads_or(ok) != 0;
 }
 
-// While waiting at the barrier of restart k: the next entry of restart k+1's
-// list (ring slot s1) for an early march, or -1.  A warp claims one index
-// (atomicAdd on the slot's head) and keeps the claim until the list holds that
-// entry; a claim still open at the release is settled by the claimer at the
-// start of restart k+1 (settle_claim).
-__device__ __forceinline__ int32_t early_entry(Ctrl* C, int32_t* list, int s1, int& claim, long long limit,
-                                               int lane) {
-    if (claim < 0) {
-        if (lane == 0) claim = atomicAdd(&C->head[s1], 1);
-        claim = __shfl_sync(0xffffffffu, claim, 0);
+// Waiting at the barrier of restart k.  One warp of the CTA at a time holds the
+// token: it polls the grid barrier and, if early work is allowed, claims the next
+// entry of restart k+1's list (one index at a time, kept in S.claim until the list
+// holds it; a claim still open at the release is settled in restart k+1).  The
+// others watch shared memory.  Returns 1: released (the CTA's state is the next
+// restart's; load(), run by one lane, reads it), 2: leave, 3: *b is a brick of
+// restart k+1 to march early.  Every wait is bounded.
+template <typename T, typename Load>
+__device__ int wait_or_work(const LoopParams<T>& P, CtaLoop& S, int k, unsigned gen, bool early, int lane, int32_t* b,
+                            Load load) {
+    Ctrl* C = P.ctrl;
+    const int s1 = (k + 1) % kRing;
+    int st = 0;
+    int32_t x = -1;
+    if (lane == 0) {
+        unsigned nap = 64;
+        for (long long it = 0;; ++it) {
+            if (vol(S.stop)) st = 2;
+            else if (vol(S.rel) != gen) st = 1;
+            else if (vol(S.token) == 0 && atomicCAS(&S.token, 0, 1) == 0) st = 3;
+            else if (it > 8 * P.wait_limit) st = 4;
+            if (st) break;
+            __nanosleep(nap);
+            if (nap < 256) nap <<= 1;
+        }
+        if (st == 3) {
+            nap = 32;
+            for (long long it = 0;; ++it) {
+                if (vol(S.rel) != gen) {
+                    st = 1;
+                    break;
+                }
+                if (ld_acquire(&C->bar_gen) != gen) {
+                    load();
+                    __threadfence_block();
+                    vol_set(S.rel, gen + 1);
+                    st = 1;
+                    break;
+                }
+                if (__ldcg(&C->status) & kStWaitTimeout) {
+                    vol_set(S.stop, 1);
+                    st = 2;
+                    break;
+                }
+                if (early) {
+                    const unsigned long long mine = static_cast<unsigned long long>(k + 1) << 32;
+                    const unsigned long long open = vol(S.claim);
+                    const int c = (open >> 32) == (mine >> 32) ? static_cast<int>(open) : atomicAdd(&C->head[s1], 1);
+                    const bool have = c < __ldcg(&C->count[s1]);
+                    vol_set(S.claim, have ? 0ull : mine | static_cast<unsigned>(c));
+                    if (have) {
+                        // (the enqueuer bumps the count, then stores the entry)
+                        x = ld_acquire(P.list[s1] + c);
+                        for (long long w = 0; x < 0 && w < P.wait_limit; ++w) {
+                            __nanosleep(32);
+                            x = ld_acquire(P.list[s1] + c);
+                        }
+                        if (x < 0) st = 4;
+                        break;
+                    }
+                }
+                if (it > P.wait_limit) {
+                    st = 4;
+                    break;
+                }
+                __nanosleep(nap);
+                if (nap < 512) nap <<= 1;
+            }
+            __threadfence_block();
+            atomicExch(&S.token, 0);
+        }
+        if (st == 4) vol_set(S.stop, 1);
     }
-    int have = 0;
-    if (lane == 0) have = claim < __ldcg(&C->count[s1]);
-    if (!__shfl_sync(0xffffffffu, have, 0)) return -1;
-    const int32_t b = take_entry(list, claim, true, limit, lane);
-    claim = -1;
-    return b < 0 ? -2 : b;
+    st = __shfl_sync(kFull, st, 0);
+    *b = __shfl_sync(kFull, x, 0);
+    if (st == 4) {
+        give_up(C, lane);
+        return 2;
+    }
+    return st;
+}
+
+// The next entry of restart k's brick list (ring slot s, S.n entries) for this
+// warp, -1 when all are handed out.  `first`: the warp's first call in the
+// restart, which settles the claim the CTA left open while waiting.
+__device__ __forceinline__ int next_entry(Ctrl* C, CtaLoop& S, int k, int s, bool first, int lane) {
+    int i = -1;
+    if (lane == 0) {
+        if (first) {
+            const unsigned long long open = vol(S.claim);
+            if (static_cast<int>(open >> 32) == k && atomicCAS(&S.claim, open, 0ull) == open) i = static_cast<int>(open);
+        }
+        if (i < 0 && vol(S.drained) != k) i = atomicAdd(&C->head[s], 1);
+        if (i >= S.n) i = -1;
+        if (i < 0) vol_set(S.drained, k);
+    }
+    return __shfl_sync(kFull, i, 0);
 }
 
 }  // namespace eikg

@@ -174,27 +174,7 @@ struct QueueRoot<double> {
     }
 };
 
-// A march's counts and the smallest and largest h/F it met, added up per warp in
-// shared memory (lane 0; the march needs its registers).
-__device__ __forceinline__ void reset_acc(MarchAcc& A) {
-    A = MarchAcc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
-}
-// ... -> the control block, at the end of the warp's share of a restart
-__device__ __forceinline__ void flush_acc8(Ctrl* C, MarchAcc& A, int lane) {
-    if (lane == 0) {
-        atomicAdd(&C->r_accepted, static_cast<unsigned long long>(A.accepted));
-        atomicAdd(&C->r_band, static_cast<unsigned long long>(A.band));
-        atomicAdd(&C->r_solves, static_cast<unsigned long long>(A.solves));
-        atomicAdd(&C->r_updates, static_cast<unsigned long long>(A.updates));
-        atomicAdd(&C->r_rounds, static_cast<unsigned long long>(A.rounds));
-        atomicMin(&C->r_rmin_bits, __float_as_uint(A.rmin));
-        atomicMax(&C->r_rmax_bits, __float_as_uint(A.rmax));
-        if (A.fallbacks) atomicAdd(&C->r_fallbacks, static_cast<unsigned long long>(A.fallbacks));
-        reset_acc(A);
-    }
-    __syncwarp();
-}
-
+// (A: the warp's statistics, in shared memory: the march needs its registers)
 template <typename T>
 __device__ void march8(const LoopParams<T>& P, const Geo& G, QueueSmem<T>& S, MarchAcc& A, int32_t b, int k, T bprev,
                        T bound, bool grow, T window, int lane, bool publish, int32_t pf = -1) {

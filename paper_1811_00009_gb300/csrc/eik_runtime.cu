@@ -108,7 +108,7 @@ struct eik_ctx {
     int64_t last_nr = 0;
     int tuned_block = 0;           // block edge picked by eik_autotune (0: not tuned)
     double tuned_stride = 0.0;     // stride picked by eik_autotune
-    int loop_grid = 0;
+    int loop_per_sm = 0;           // CTAs of the restart loop that fit an SM
     int sms = 0;
     eik_params params{};
     eikg::Ctrl host_ctrl{};
@@ -346,7 +346,7 @@ eik_status eik_create(eik_ctx** out, const int32_t dims[3], double h, const void
     e = (c->prec == EIK_FP32) ? eikg::loop_occupancy<float>(&per_sm) : eikg::loop_occupancy<double>(&per_sm);
     if (e != cudaSuccess || per_sm < 1)
         return bail(EIK_ECUDA, std::string("eik_create: occupancy query: ") + cudaGetErrorString(e));
-    c->loop_grid = per_sm * c->sms;
+    c->loop_per_sm = per_sm;
     // every context starts with the shipped schedule network (eik_set_schedule replaces or unloads it)
     static_assert(EIK_SCHED_DEFAULT_COUNT == eikg::kParams, "shipped weights match the network");
     e = cudaMalloc(&c->d_mlp, sizeof(float) * eikg::kParams);
@@ -674,7 +674,8 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
             return EIK_OK;
         }
         if (P.loop_events[0]) EIK_CK(c, cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[0]), s));
-        EIK_CK(c, eikg::launch_restart_loop<T>(L, c->loop_grid, s));
+        EIK_CK(c, eikg::launch_restart_loop<T>(
+            L, eikh::restart_loop_ctas(c->loop_per_sm, c->sms, c->nbricks, P.block_dim), s));
         if (P.loop_events[1]) EIK_CK(c, cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[1]), s));
     }
     if (nfix > 0)
@@ -1066,8 +1067,9 @@ eik_status eik_slab_restart(eik_ctx* c, int64_t* pending) {
     if (!c) return fail(nullptr, EIK_EINVAL, "eik_slab_restart: ctx is NULL");
     if (!c->slab_running) return fail(c, EIK_ESTATE, "eik_slab_restart: no sharded solve begun (eik_slab_begin)");
     EIK_CK(c, cudaMemsetAsync(&c->ctrl->done, 0, sizeof(int32_t), c->stream));
-    if (c->prec == EIK_FP32) EIK_CK(c, eikg::launch_restart_loop<float>(c->lp_f, c->loop_grid, c->stream));
-    else EIK_CK(c, eikg::launch_restart_loop<double>(c->lp_d, c->loop_grid, c->stream));
+    const int ctas = eikh::restart_loop_ctas(c->loop_per_sm, c->sms, c->nbricks, 8);
+    if (c->prec == EIK_FP32) EIK_CK(c, eikg::launch_restart_loop<float>(c->lp_f, ctas, c->stream));
+    else EIK_CK(c, eikg::launch_restart_loop<double>(c->lp_d, ctas, c->stream));
     return slab_pending(c, pending);
 }
 
