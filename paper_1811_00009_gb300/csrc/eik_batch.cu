@@ -17,7 +17,7 @@
 #include "eik.h"
 #include "eik_host.h"
 #include "eik_internal.cuh"
-#include "eik_march8.cuh"
+#include "eik_march16.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -114,14 +114,13 @@ __device__ void load_batch_restart(const LoopParams<T>& P, CtaLoop& S) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_loop(LoopParams<T> P) {
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_loop(const __grid_constant__ LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
     __shared__ CtaLoop S;
     __shared__ MarchAcc s_acc[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
     QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
     Ctrl* C = P.ctrl;
     MarchAcc& A = s_acc[warp];
@@ -156,7 +155,6 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_l
             if (!cta_go(C, true, lane, &s_arrived)) return;
             {
                 const int n = __ldcg(&C->gcount[s]);
-                MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
                 bool grouped = false;
                 for (;;) {
                     __syncthreads();
@@ -173,25 +171,13 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_l
                     const Geo G{D.BX, D.BY, D.BZ, D.boff, D.GX, D.GY, D.goff, 2u, D.div_x, D.div_xy};
                     const int gl = g - D.goff;
                     const int gx = gl % D.GX, gy = (gl / D.GX) % D.GY, gz = gl / (D.GX * D.GY);
-                    const int bx = 2 * gx + (warp & 1), by = 2 * gy + ((warp >> 1) & 1), bz = 2 * gz + (warp >> 2);
-                    const bool in = bx < D.BX && by < D.BY && bz < D.BZ;
-                    const int32_t b = in ? D.boff + (bz * D.BY + by) * D.BX + bx : -1;
-                    unsigned gmask = 0;
-                    if (in) {
-                        if (warp & 1) gmask |= 1u;
-                        else if (bx + 1 < D.BX) gmask |= 2u;
-                        if (warp & 2) gmask |= 4u;
-                        else if (by + 1 < D.BY) gmask |= 8u;
-                        if (warp & 4) gmask |= 16u;
-                        else if (bz + 1 < D.BZ) gmask |= 32u;
-                    }
-                    march_group<T>(P, G, SW, warp, b, gmask, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
-                                   pick<T>(P.window, P.window_f), lane, acc, P.early != 0);
+                    march16<T>(P, G, A, gx, gy, gz, k, batch_bound(P, sv, k - 1), batch_bound(P, sv, k), true,
+                                   pick<T>(P.window, P.window_f));
                     if (threadIdx.x == 0) atomicMax(P.last_k + sv, k);
                     grouped = true;
                 }
                 if (grouped) {
-                    flush_acc(C, acc, lane);
+                    any = true;
                     init_queue_smem(SQ[warp], lane);              // (the groups' tiles overlay it)
                 }
             }
@@ -279,7 +265,7 @@ __global__ void k_owner(int32_t* __restrict__ tab, int64_t n, const int32_t* __r
 
 template <typename T>
 size_t batch_smem_bytes() {
-    return std::max(sizeof(WarpSmem<T>), sizeof(QueueSmem<T>)) * kWarps;
+    return std::max(sizeof(GroupSmem<T>), sizeof(QueueSmem<T>) * kWarps);
 }
 
 template <typename T>

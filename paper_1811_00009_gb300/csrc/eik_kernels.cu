@@ -7,7 +7,7 @@
 // the start of the next march (see eik_internal.cuh for the double-copy
 // layout that makes this race-free, the argument of Sec. 2.7).
 #include "eik_internal.cuh"
-#include "eik_march8.cuh"
+#include "eik_march16.cuh"
 #include "eik_mlp.cuh"
 
 #include <algorithm>
@@ -257,7 +257,7 @@ __device__ void load_restart(const LoopParams<T>& P, CtaLoop& S) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart_loop(LoopParams<T> P) {
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart_loop(const __grid_constant__ LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
@@ -265,7 +265,6 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
     __shared__ MarchAcc s_acc[kWarps];
     __shared__ WarpLoop s_warp[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpSmem<T>* SW = reinterpret_cast<WarpSmem<T>*>(smem_raw);
     QueueSmem<T>* SQ = reinterpret_cast<QueueSmem<T>*>(smem_raw);
     Ctrl* C = P.ctrl;
     MarchAcc& A = s_acc[warp];
@@ -308,8 +307,6 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
                                                P.glist[s], s, k, P.BX, P.BY, P.GX, P.GY, P.wait_limit);
             if (!cta_go(C, ok, lane, &s_arrived)) return;
             // one CTA per group of 2x2x2 bricks
-            MarchAcc acc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
-            bool grouped = false;
             const int n = __ldcg(&C->gcount[s]);
             for (;;) {
                 __syncthreads();
@@ -322,23 +319,10 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
                 const int g = s_item;
                 if (g < 0) break;
                 const int gx = g % P.GX, gy = (g / P.GX) % P.GY, gz = g / (P.GX * P.GY);
-                const int bx = 2 * gx + (warp & 1), by = 2 * gy + ((warp >> 1) & 1), bz = 2 * gz + (warp >> 2);
-                const bool in = bx < P.BX && by < P.BY && bz < P.BZ;
-                const int32_t b = in ? (bz * P.BY + by) * P.BX + bx : -1;
-                unsigned gmask = 0;
-                if (in) {
-                    if (warp & 1) gmask |= 1u;                     // -x neighbour in the group
-                    else if (bx + 1 < P.BX) gmask |= 2u;           // +x
-                    if (warp & 2) gmask |= 4u;
-                    else if (by + 1 < P.BY) gmask |= 8u;
-                    if (warp & 4) gmask |= 16u;
-                    else if (bz + 1 < P.BZ) gmask |= 32u;
-                }
-                march_group<T>(P, G, SW, warp, b, gmask, k, pick<T>(S.bprev, S.bprev_f), pick<T>(S.bound, S.bound_f),
-                               S.grow != 0, pick<T>(P.window, P.window_f), lane, acc, S.early != 0);
-                grouped = true;
+                march16<T>(P, G, A, gx, gy, gz, k, pick<T>(S.bprev, S.bprev_f), pick<T>(S.bound, S.bound_f),
+                               S.grow != 0, pick<T>(P.window, P.window_f));
+                any = true;
             }
-            if (grouped) flush_acc(C, acc, lane);
             init_queue_smem(SQ[warp], lane);          // (the groups' tiles overlay it)
         }
         // One warp per 8^3 brick: this restart's list, then -- once arrived at
@@ -703,7 +687,7 @@ cudaError_t launch_slab_import(T* slot, unsigned long long* ups, unsigned long l
 
 template <typename T>
 size_t loop_smem_bytes() {
-    return std::max(sizeof(WarpSmem<T>), sizeof(QueueSmem<T>)) * kWarps;
+    return std::max(sizeof(GroupSmem<T>), sizeof(QueueSmem<T>) * kWarps);
 }
 
 template <typename T>

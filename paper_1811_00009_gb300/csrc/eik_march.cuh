@@ -331,45 +331,10 @@ __device__ __forceinline__ float pick<float>(double, float f) { return f; }
 template <>
 __device__ __forceinline__ double pick<double>(double d, float) { return d; }
 
-template <typename T>
-struct RootOf;
-template <>
-struct RootOf<float> {
-    static __device__ __forceinline__ float go(float a, float b, float c, float r, float tau, int& fb) {
-        return upwind_root_f32(a, b, c, r, tau, fb);
-    }
-};
-template <>
-struct RootOf<double> {
-    static __device__ __forceinline__ double go(double a, double b, double c, double r, float, int&) {
-        return upwind_root(a, b, c, r);
-    }
-};
-
-// Per-warp shared memory.
-constexpr int kBandCap = 896;      // 512 interior + 384 ghost nodes: every node at most once
-
-template <typename T>
-struct __align__(16) WarpSmem {
-    T psi[1000];            // brick plus one ghost layer, index ((z+1)*10 + (y+1))*10 + (x+1)
-    T r[kBrick];            // h/F, brick index
-    uint16_t band[kBandCap];// the narrow band: halo indices of the pending nodes
-    uint16_t list[kBrick];  // nodes to re-solve in the current round (halo index)
-    uint32_t mark[32];      // one warp: halo bit vector of the nodes accepted in this round;
-                            // group of warps: bit per brick node, neighbour of a node accepted this round
-    uint32_t upd[16];       // bit per brick node: lowered in this march (Upsilon)
-    uint32_t fxob[16];      // bit per brick node: fixed, barrier or padding node (never solved)
-};
-
 // Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) of global memory
 // into L2, without a destination or a completion to wait for.
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ int halo_of(int p) {
-    const int x = p & 7, y = (p >> 3) & 7, z = p >> 6;
-    return ((z + 1) * 10 + (y + 1)) * 10 + (x + 1);
 }
 
 template <typename T>
@@ -420,21 +385,6 @@ __device__ __forceinline__ void store8<double>(double* g, const double* v) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) reinterpret_cast<double2*>(g)[i] = make_double2(v[2 * i], v[2 * i + 1]);
 }
-template <typename T>
-__device__ __forceinline__ void load2_cg(const T* g, T& a, T& b);
-template <>
-__device__ __forceinline__ void load2_cg<float>(const float* g, float& a, float& b) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(g));
-    a = v.x;
-    b = v.y;
-}
-template <>
-__device__ __forceinline__ void load2_cg<double>(const double* g, double& a, double& b) {
-    const double2 v = __ldcg(reinterpret_cast<const double2*>(g));
-    a = v.x;
-    b = v.y;
-}
-
 // Minimum over the warp of values that are >= 0 (+inf allowed): the bits of
 // non-negative IEEE numbers order like unsigned integers, so one integer
 // reduction (two for FP64: high words, then low words among the lanes holding
@@ -460,12 +410,6 @@ __device__ __forceinline__ T warp_max(T v) {            // (values >= 0)
         return v;
     }
 }
-__device__ __forceinline__ unsigned long long warp_or64(unsigned long long v) {
-    const unsigned lo = __reduce_or_sync(kFull, static_cast<unsigned>(v));
-    const unsigned hi = __reduce_or_sync(kFull, static_cast<unsigned>(v >> 32));
-    return (static_cast<unsigned long long>(hi) << 32) | lo;
-}
-
 struct MarchAcc {
     unsigned accepted;                       // per lane
     unsigned band;                           // counted on lane 0
@@ -474,22 +418,6 @@ struct MarchAcc {
     unsigned solves, rounds;                 // the same on every lane (one restart of one warp)
     float rmin, rmax;                        // the same on every lane
 };
-
-// Face-local element u of face f (x faces: u = z*8+y, y faces: u = z*8+x,
-// z faces: u = y*8+x): halo index of the ghost node beyond face f, and halo
-// index of the brick's own boundary node on face f.
-__device__ __forceinline__ int face_ghost_halo(int f, int u) {
-    const int a = u & 7, c = u >> 3;
-    if (f < 2) return ((c + 1) * 10 + (a + 1)) * 10 + (f == 0 ? 0 : 9);
-    if (f < 4) return ((c + 1) * 10 + (f == 2 ? 0 : 9)) * 10 + (a + 1);
-    return ((f == 4 ? 0 : 9) * 10 + (c + 1)) * 10 + (a + 1);
-}
-__device__ __forceinline__ int face_own_halo(int f, int u) {
-    const int a = u & 7, c = u >> 3;
-    if (f < 2) return ((c + 1) * 10 + (a + 1)) * 10 + (f == 0 ? 1 : 8);
-    if (f < 4) return ((c + 1) * 10 + (f == 2 ? 1 : 8)) * 10 + (a + 1);
-    return ((f == 4 ? 1 : 8) * 10 + (c + 1)) * 10 + (a + 1);
-}
 
 // Where a grid sits in the work space of a launch: its bricks are the global
 // indices [boff, boff + BX*BY*BZ), its 2x2x2 groups [goff, goff + GX*GY*GZ).
@@ -536,431 +464,6 @@ __device__ __forceinline__ void enqueue_next(const LoopParams<T>& P, const Geo& 
     }
 }
 
-// March_Narrow_Band (Alg. 4) of brick b at restart k, with the exchange of
-// Alg. 5 for its ghost layer done first from the neighbours' copies as of the
-// end of restart k-1.
-//
-// The eight warps of the
-// CTA march the 2x2x2 bricks of one 16^3 block together (warp w holds brick
-// (w & 1, (w >> 1) & 1, w >> 2) of the group; b < 0 for a brick outside the
-// grid, whose warp only takes part in the barriers).  The rounds then share
-// one acceptance threshold, an accepted node marks the neighbouring warp's
-// nodes across internal faces, and after every phase each warp refreshes its
-// ghost layer on internal faces from the neighbouring warp's tile, so
-// information crosses the internal faces within the restart as it does inside
-// one block of the paper.
-template <typename T>
-__device__ void march_group(const LoopParams<T>& P, const Geo& G, WarpSmem<T>* SW, int warp, int32_t b, unsigned gmask,
-                      int k, T bprev, T bound, bool grow, T window, int lane, MarchAcc& acc, bool publish) {
-    __shared__ T s_wmin[kWarps];
-    __shared__ T s_bmin[2][kWarps];            // group rounds: band minima, by round parity
-    WarpSmem<T>& S = SW[warp];
-    const T INF = Num<T>::inf();
-    const bool present = b >= 0;
-    const int y = lane & 7, zp = lane >> 3, z0 = 2 * zp;
-    const int BX = G.BX, BY = G.BY, BZ = G.BZ;
-    const int bb = present ? b : G.boff;                         // global index; coordinates are local
-    const int bl = bb - G.boff;
-    const int bx = bl % BX, by = (bl / BX) % BY, bz = bl / (BX * BY);
-    const int pbase = (z0 * 8 + y) * 8;                          // brick index of (0, y, z0)
-    const int hbase = ((z0 + 1) * 10 + (y + 1)) * 10 + 1;       // halo index of (0, y, z0)
-    const unsigned lt = (1u << lane) - 1u;
-
-    int nbr[6];
-    nbr[0] = bx > 0 ? bb - 1 : -1;
-    nbr[1] = bx < BX - 1 ? bb + 1 : -1;
-    nbr[2] = by > 0 ? bb - BX : -1;
-    nbr[3] = by < BY - 1 ? bb + BX : -1;
-    nbr[4] = bz > 0 ? bb - BX * BY : -1;
-    nbr[5] = bz < BZ - 1 ? bb + BX * BY : -1;
-
-    unsigned long long st = kUntouched;
-    unsigned FXOB = 0xFFFFu;
-    T rlo = INF, rhi = 0;
-    int n = 0;
-    if (present) {
-        // ---- load phase 1 (independent loads): stamps of the brick and its six
-        // neighbours, and h/F of this lane's two rows
-        st = __ldcg(P.stamp + b);
-        unsigned long long wst[6];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) wst[f] = nbr[f] >= 0 ? __ldcg(P.stamp + nbr[f]) : kUntouched;
-        // fixed nodes (r < 0) and barrier/padding nodes (r = +inf) are never solved
-        FXOB = 0;
-        {
-            T row[8];
-            const T* rs = P.rr + static_cast<int64_t>(b) * kBrick;
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                load8_ro(rs + pbase + 64 * s, row);
-                store8(S.r + pbase + 64 * s, row);
-#pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const T r = row[x];
-                    if (!(r > 0) || !(r < INF)) FXOB |= 1u << (8 * s + x);
-                    else {
-                        rlo = vmin(rlo, r);
-                        rhi = vmax(rhi, r);
-                    }
-                }
-            }
-        }
-        // ---- load phase 2: the brick's latest copy, and the ghost layer: the
-        // neighbours' faces as of the end of restart k-1 with their Upsilon masks
-        // (Alg. 5).  A neighbour that already marched in this restart is read from
-        // its other copy.
-        unsigned long long fups[6];
-        T fv0[6], fv1[6];
-        const int u = 2 * lane;                                   // face-local index of this lane's pair
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            const unsigned long long w = wst[f];
-            int sl = -1, written = -1;
-            if (w != kUntouched) {
-                if (stamp_latest(w) >= k) {
-                    written = stamp_other(w);
-                    sl = (written == static_cast<int>(kNever)) ? -1 : (stamp_copy(w) ^ 1);
-                } else {
-                    written = stamp_latest(w);
-                    sl = stamp_copy(w);
-                }
-            }
-            fups[f] = (sl >= 0 && written == k - 1)
-                          ? __ldcg(P.ups + (static_cast<int64_t>(nbr[f]) * 2 + sl) * 6 + (f ^ 1))
-                          : 0ull;
-            fv0[f] = INF;
-            fv1[f] = INF;
-            if (sl >= 0) {
-                const T* src = P.slot + (static_cast<int64_t>(nbr[f]) * 2 + sl) * kSlot;
-                int off;
-                if (f == 0) off = kXF7 + u;
-                else if (f == 1) off = kXF0 + u;
-                else if (f == 2) off = ((u >> 3) * 8 + 7) * 8 + (u & 7);
-                else if (f == 3) off = ((u >> 3) * 8 + 0) * 8 + (u & 7);
-                else if (f == 4) off = 7 * 64 + u;
-                else off = u;
-                load2_cg(src + off, fv0[f], fv1[f]);
-            }
-        }
-        // ---- the band at the start of the march (marked as the values land in
-        // shared memory): the brick's finite nodes above the previous bound, and
-        // the ghost nodes that are above it or that the neighbour lowered in
-        // restart k-1 (Upsilon) -- the heap contents of Alg. 4 after Alg. 5.
-        // Lane L marks its two rows (bits 0-15 of B) and face-local nodes 2L and
-        // 2L+1 of each face (bits 2f and 2f+1 of G).
-        unsigned B = 0, G = 0;
-        if (st == kUntouched) {
-#pragma unroll
-            for (int x = 0; x < 8; ++x) S.psi[hbase + x] = INF, S.psi[hbase + 100 + x] = INF;
-        } else {
-            const T* src = P.slot + (static_cast<int64_t>(b) * 2 + stamp_copy(st)) * kSlot;
-            T row[8], row1[8];
-            load8_cg(src + pbase, row);
-            load8_cg(src + pbase + 64, row1);
-#pragma unroll
-            for (int x = 0; x < 8; ++x) {
-                const T v0 = row[x], v1 = row1[x];
-                const bool b0 = v0 < INF && v0 > bprev, b1 = v1 < INF && v1 > bprev;
-                S.psi[hbase + x] = b0 ? -v0 : v0;
-                S.psi[hbase + 100 + x] = b1 ? -v1 : v1;
-                B |= (b0 ? 1u : 0u) << x;
-                B |= (b1 ? 1u : 0u) << (8 + x);
-            }
-        }
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            const int h0 = face_ghost_halo(f, u);
-            const T g0 = fv0[f], g1 = fv1[f];
-            const bool b0 = g0 < INF && (((fups[f] >> u) & 1ull) || g0 > bprev);
-            const bool b1 = g1 < INF && (((fups[f] >> (u + 1)) & 1ull) || g1 > bprev);
-            S.psi[h0] = b0 ? -g0 : g0;
-            S.psi[h0 + (f < 2 ? 10 : 1)] = b1 ? -g1 : g1;
-            G |= ((b0 ? 1u : 0u) | (b1 ? 2u : 0u)) << (2 * f);
-        }
-        // ---- the band as a list shared by the warp (one entry per pending node)
-        const int cnt = __popc(B) + __popc(G);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        n = __shfl_sync(kFull, incl, 31);
-        int off = incl - cnt;
-        for (unsigned m = B; m; m &= m - 1) {
-            const int j = __ffs(m) - 1;
-            S.band[off++] = static_cast<uint16_t>(hbase + (j >> 3) * 100 + (j & 7));
-        }
-        for (unsigned m = G; m; m &= m - 1) {
-            const int j = __ffs(m) - 1, f = j >> 1;
-            S.band[off++] = static_cast<uint16_t>(face_ghost_halo(f, u) + ((j & 1) ? (f < 2 ? 10 : 1) : 0));
-        }
-    }
-    if (lane < 16) {
-        S.mark[lane] = 0u;
-        S.upd[lane] = 0u;
-        S.fxob[lane] = 0u;
-    }
-    __syncwarp();
-    if (FXOB & 0xFFu) atomicOr(&S.fxob[pbase >> 5], (FXOB & 0xFFu) << (pbase & 31));
-    if (FXOB >> 8) atomicOr(&S.fxob[(pbase + 64) >> 5], (FXOB >> 8) << ((pbase + 64) & 31));
-
-    const T rmin_b = warp_min_nn(rlo);
-    if (present) {
-        acc.rmin = fminf(acc.rmin, static_cast<float>(rmin_b));
-        acc.rmax = fmaxf(acc.rmax, static_cast<float>(warp_max(rhi)));
-    }
-    // one window for the group: omega times the smallest h/F of its bricks
-    if (lane == 0) s_wmin[warp] = rmin_b;
-    __syncthreads();
-    T w = s_wmin[0];
-#pragma unroll
-    for (int i = 1; i < kWarps; ++i) w = vmin(w, s_wmin[i]);
-    w = window * w;
-    __syncthreads();
-    const float tau = static_cast<float>(P.fallback_tau);
-
-    // ghost layer on internal faces <- the neighbouring warps' boundary nodes
-    auto refresh_internal = [&]() {
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            if (!((gmask >> f) & 1u)) continue;
-            const WarpSmem<T>& NB = SW[warp ^ (1 << (f >> 1))];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int uu = 2 * lane + e;
-                S.psi[face_ghost_halo(f, uu)] = NB.psi[face_own_halo(f ^ 1, uu)];
-            }
-        }
-        __syncwarp();
-    };
-
-    // Alg. 3 for each listed node (halo index), 32 at a time; new values land
-    // after the reads.  A lowered node is tagged BAND (Alg. 2) and joins the band
-    // unless it is in it already.  Returns this lane's smallest lowered value.
-    auto solve_list = [&](int total) -> T {
-        T smin = INF;
-        for (int base = 0; base < total; base += 32) {
-            const int idx = base + lane;
-            bool imp = false, known = false;
-            T xn = 0;
-            int hq = 0, q = 0;
-            if (idx < total) {
-                hq = S.list[idx];
-                // brick index of the halo position: z = hq / 100, y = (hq % 100) / 10 (exact for hq < 1000)
-                const int hz = (hq * 41) >> 12, rem = hq - 100 * hz, hy = (rem * 103) >> 10;
-                q = hz * 64 + hy * 8 + (rem - 10 * hy) - 73;
-                const T cur = S.psi[hq];
-                const T c = vabs(cur);
-                known = !sgn(cur);
-                // KNOWN neighbours below the node's current value (Alg. 3's test): as
-                // unsigned bit patterns every KNOWN (sign clear) value orders as its
-                // value and every BAND value (sign set) lies above any KNOWN one
-                // (per axis: the smaller bit pattern of the two neighbours is the
-                // smaller KNOWN value if either is KNOWN; it counts if below c)
-                const auto cb = ubits(c);
-                auto axis = [&](T a, T b) -> T {
-                    const auto ua = ubits(a), ub = ubits(b);
-                    const auto m = ua < ub ? ua : ub;
-                    return m < cb ? from_bits(m) : INF;
-                };
-                T mx = axis(S.psi[hq - 1], S.psi[hq + 1]);
-                T my = axis(S.psi[hq - 10], S.psi[hq + 10]);
-                T mz = axis(S.psi[hq - 100], S.psi[hq + 100]);
-                // reorder psi_1 <= psi_2 <= psi_3
-                T lo = vmin(mx, my), hi = vmax(mx, my);
-                T a0 = vmin(lo, mz);
-                T t1 = vmax(lo, mz);
-                T a1 = vmin(hi, t1), a2 = vmax(hi, t1);
-                if (vlt(a0, INF)) {
-                    xn = RootOf<T>::go(a0, a1, a2, S.r[q], tau, acc.fallbacks);
-                    imp = vlt(xn, c);
-                }
-            }
-            __syncwarp();
-            const bool add = imp && known;
-            const unsigned am = __ballot_sync(kFull, add);
-            if (imp) {
-                S.psi[hq] = -xn;
-                atomicOr(&S.upd[q >> 5], 1u << (q & 31));
-                smin = vmin(smin, xn);
-            }
-            if (add) S.band[n + __popc(am & lt)] = static_cast<uint16_t>(hq);
-            n += __popc(am);
-            acc.updates += imp ? 1u : 0u;
-            __syncwarp();
-        }
-        return smin;
-    };
-    // lane-distributed bit set -> S.list (ascending), returns the entry count
-    auto compact = [&](unsigned bits, int first) -> int {
-        const int cnt = __popc(bits);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        int off = incl - cnt;
-        for (unsigned m = bits; m; m &= m - 1) S.list[off++] = static_cast<uint16_t>(first + __ffs(m) - 1);
-        __syncwarp();
-        return __shfl_sync(kFull, incl, 31);
-    };
-
-    // ---- rounds of windowed ordered acceptance (Alg. 4)
-    int rounds = 0;
-    for (;;) {
-        T lmin = INF;
-        for (int i = lane; i < n; i += 32) lmin = vmin(lmin, vabs(S.psi[S.band[i]]));
-        T mn = warp_min_nn(lmin);
-        // (two buffers by round parity: the barriers later in the round order
-        // these reads before the writes two rounds on, so one barrier suffices)
-        T* bm = s_bmin[rounds & 1];
-        if (lane == 0) bm[warp] = mn;
-        __syncthreads();
-        T g = bm[0];
-#pragma unroll
-        for (int i = 1; i < kWarps; ++i) g = vmin(g, bm[i]);
-        mn = g;
-        if (!(mn < INF) || !(mn <= bound)) break;   // band empty, or its minimum above the bound
-        if (++rounds > kRoundCap) {
-            atomicOr(&P.ctrl->status, kStRoundCap);
-            break;
-        }
-        const T thr = vmin(mn + w, bound);
-        // accept (Remove_Min of a window), keep the rest of the band in order,
-        // and mark the accepted nodes' neighbours (Alg. 2), across internal
-        // faces in the neighbouring warp's tile
-        int kept = 0;
-        for (int base = 0; base < n; base += 32) {
-            const int i = base + lane;
-            int hh = 0;
-            bool keep = false, take = false;
-            if (i < n) {
-                hh = S.band[i];
-                const T v = vabs(S.psi[hh]);
-                if (!vlt(thr, v)) {
-                    take = true;
-                    S.psi[hh] = v;
-                } else {
-                    keep = true;
-                }
-            }
-            const unsigned km = __ballot_sync(kFull, keep);
-            if (keep) S.band[kept + __popc(km & lt)] = static_cast<uint16_t>(hh);
-            kept += __popc(km);
-            acc.accepted += take ? 1u : 0u;
-            if (take) {
-                const int px = hh % 10 - 1, py = (hh / 10) % 10 - 1, pz = hh / 100 - 1;
-                const T va = S.psi[hh];                 // (accepted: sign clear)
-                auto cand = [&](int x, int yy, int z) {
-                    const bool ix = static_cast<unsigned>(x) < 8u, iy = static_cast<unsigned>(yy) < 8u,
-                               iz = static_cast<unsigned>(z) < 8u;
-                    if (ix && iy && iz) {
-                        const int q = (z * 8 + yy) * 8 + x;
-                        atomicOr(&S.mark[q >> 5], 1u << (q & 31));
-                    } else {
-                        int f = -1;
-                        if (!ix && iy && iz) f = (x < 0) ? 0 : 1;
-                        else if (ix && !iy && iz) f = (yy < 0) ? 2 : 3;
-                        else if (ix && iy && !iz) f = (z < 0) ? 4 : 5;
-                        if (f >= 0 && ((gmask >> f) & 1u)) {
-                            const int q = (((z & 7) * 8) + (yy & 7)) * 8 + (x & 7);
-                            atomicOr(&SW[warp ^ (1 << (f >> 1))].mark[q >> 5], 1u << (q & 31));
-                        }
-                    }
-                };
-                // only neighbours above the accepted value can be lowered by it (beyond
-                // an internal face the ghost layer's copy: never below the node itself)
-                const int pi = ((pz + 1) * 10 + (py + 1)) * 10 + px + 1;
-                if (px > -1 && vlt(va, vabs(S.psi[pi - 1]))) cand(px - 1, py, pz);
-                if (px < 8 && vlt(va, vabs(S.psi[pi + 1]))) cand(px + 1, py, pz);
-                if (py > -1 && vlt(va, vabs(S.psi[pi - 10]))) cand(px, py - 1, pz);
-                if (py < 8 && vlt(va, vabs(S.psi[pi + 10]))) cand(px, py + 1, pz);
-                if (pz > -1 && vlt(va, vabs(S.psi[pi - 100]))) cand(px, py, pz - 1);
-                if (pz < 8 && vlt(va, vabs(S.psi[pi + 100]))) cand(px, py, pz + 1);
-            }
-        }
-        n = kept;
-        __syncthreads();
-        refresh_internal();
-        __syncthreads();
-        // candidates (brick bits, 16 per lane) -> list of halo indices; never-solved nodes dropped
-        const unsigned word = S.mark[lane >> 1] & ~S.fxob[lane >> 1];
-        const unsigned wd = (lane & 1) ? (word >> 16) : (word & 0xFFFFu);
-        __syncwarp();
-        if (lane < 16) S.mark[lane] = 0u;
-        const int total = compact(wd, 16 * lane);   // brick indices
-        for (int i = lane; i < total; i += 32) S.list[i] = static_cast<uint16_t>(halo_of(S.list[i]));
-        __syncwarp();
-        acc.solves += total;
-        solve_list(total);
-        // no barrier or refresh here: the next round's first barrier orders these
-        // writes before any other warp's marks and reads, and the ghost layer is
-        // refreshed after the next accept pass, before any solve reads it
-    }
-    acc.rounds += rounds;
-    __syncthreads();
-    if (!present) return;
-
-    // ---- Upsilon: own face nodes lowered in this march, per face (face-local bit
-    // masks); none on internal faces of a group, whose neighbours saw them live
-    const unsigned U = ((S.upd[pbase >> 5] >> (pbase & 31)) & 0xFFu) |
-                       (((S.upd[(pbase + 64) >> 5] >> ((pbase + 64) & 31)) & 0xFFu) << 8);
-    unsigned long long um[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-    // A march that lowered no value leaves the brick as its latest copy holds it
-    // (which nodes are accepted follows from the bounds), so it writes nothing:
-    // readers keep taking that copy, and its Upsilon masks, written in an earlier
-    // restart, are not applied again.
-    if (__any_sync(kFull, U != 0u)) {
-        um[0] = (static_cast<unsigned long long>(U & 1u) << (z0 * 8 + y)) |
-                (static_cast<unsigned long long>((U >> 8) & 1u) << ((z0 + 1) * 8 + y));
-        um[1] = (static_cast<unsigned long long>((U >> 7) & 1u) << (z0 * 8 + y)) |
-                (static_cast<unsigned long long>((U >> 15) & 1u) << ((z0 + 1) * 8 + y));
-        um[2] = (y == 0) ? (static_cast<unsigned long long>(U & 0xFFFFu) << (z0 * 8)) : 0ull;
-        um[3] = (y == 7) ? (static_cast<unsigned long long>(U & 0xFFFFu) << (z0 * 8)) : 0ull;
-        um[4] = (zp == 0) ? (static_cast<unsigned long long>(U & 0xFFu) << (y * 8)) : 0ull;
-        um[5] = (zp == 3) ? (static_cast<unsigned long long>((U >> 8) & 0xFFu) << (y * 8)) : 0ull;
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            um[f] = warp_or64(um[f]);
-            if (((gmask >> f) & 1u)) um[f] = 0ull;
-        }
-
-        // ---- write the other copy, then publish it
-        const int ns = (st == kUntouched) ? 0 : (stamp_copy(st) ^ 1);
-        T* dst = P.slot + (static_cast<int64_t>(b) * 2 + ns) * kSlot;
-        {
-            T row[8];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-#pragma unroll
-                for (int x = 0; x < 8; ++x) row[x] = vabs(S.psi[hbase + 100 * s + x]);
-                store8(dst + pbase + 64 * s, row);
-                dst[kXF0 + (z0 + s) * 8 + y] = row[0];
-                dst[kXF7 + (z0 + s) * 8 + y] = row[7];
-            }
-        }
-        if (lane < 6) P.ups[(static_cast<int64_t>(b) * 2 + ns) * 6 + lane] = um[lane];
-        // No fence: nobody reads this copy before the grid barrier that ends the
-        // restart (a reader that sees the new stamp takes the other copy).
-        if (lane == 0)
-            P.stamp[b] = make_stamp(k, st == kUntouched ? static_cast<int>(kNever) : stamp_latest(st), ns);
-    }
-
-    // ---- activation for restart k+1 (A of Alg. 4/5, C of Alg. 4)
-    // (once the bound has reached width_band, pending nodes above it stay tentative: Alg. 6's A flag)
-    if (lane == 6 && n > 0 && grow) enqueue_next(P, G, k, b);
-    if (lane < 6 && um[lane] != 0ull && nbr[lane] >= 0) enqueue_next(P, G, k, nbr[lane]);
-    if (lane == 0) acc.band += n;
-    // publish: the brick's restart-k march has finished (read by early marches
-    // of its neighbours; the release store orders the warp's writes above it)
-    if (publish) {
-        __syncwarp();
-        if (lane == 0) st_release(P.done + b, k);
-    }
-}
-
 // At the start of restart k: every thread of the launch clears its share of the
 // brick list restart k-1 used (ring slot (k-1) mod kRing, `used` entries),
 // coalesced.  The slot is next written in restart k+1 (by early marches of
@@ -1001,25 +504,6 @@ __device__ bool wait_ready(const LoopParams<T>& P, const Geo& G, int32_t b, int 
     }
     __syncwarp();
     return true;
-}
-
-// This warp's statistics of the restart, kept in registers -> the control block.
-__device__ __forceinline__ void flush_acc(Ctrl* C, MarchAcc& acc, int lane) {
-    const unsigned acc_a = __reduce_add_sync(0xffffffffu, acc.accepted);
-    const unsigned acc_b = __reduce_add_sync(0xffffffffu, acc.band);
-    const int fb = __reduce_add_sync(0xffffffffu, acc.fallbacks);
-    const unsigned upd = __reduce_add_sync(0xffffffffu, acc.updates);
-    if (lane == 0) {
-        atomicAdd(&C->r_accepted, static_cast<unsigned long long>(acc_a));
-        atomicAdd(&C->r_band, static_cast<unsigned long long>(acc_b));
-        atomicAdd(&C->r_solves, static_cast<unsigned long long>(acc.solves));
-        atomicAdd(&C->r_updates, static_cast<unsigned long long>(upd));
-        atomicAdd(&C->r_rounds, static_cast<unsigned long long>(acc.rounds));
-        atomicMin(&C->r_rmin_bits, __float_as_uint(acc.rmin));
-        atomicMax(&C->r_rmax_bits, __float_as_uint(acc.rmax));
-        if (fb) atomicAdd(&C->r_fallbacks, static_cast<unsigned long long>(fb));
-    }
-    acc = MarchAcc{0u, 0u, 0, 0u, 0u, 0u, __int_as_float(0x7f800000), 0.0f};
 }
 
 // State of the restart loop shared by a CTA's warps.  The control block sits in
