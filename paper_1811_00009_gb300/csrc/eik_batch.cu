@@ -113,7 +113,9 @@ __device__ void load_batch_restart(const LoopParams<T>& P, CtaLoop& S) {
     S.gen = gen;
 }
 
-template <typename T>
+// (GROUPS: some grids have 16^3 blocks.  A template: with march16 in the loop the
+// compiler has fewer registers for march8.)
+template <typename T, bool GROUPS>
 __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_loop(const __grid_constant__ LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
@@ -148,10 +150,10 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_batch_l
         const int k = S.k;
         const int s = k % kRing;
         const unsigned gen = S.gen;
-        clear_used_slot(P, k, S.used);
+        clear_used_slot(P.list[(k + kRing - 1) % kRing], S.used);
         // ---- 16^3 blocks (if any grid has them): one CTA per group of 2x2x2 bricks
         // (the CTA goes on only as a whole)
-        if (P.groups) {
+        if (GROUPS) {
             if (!cta_go(C, true, lane, &s_arrived)) return;
             {
                 const int n = __ldcg(&C->gcount[s]);
@@ -269,20 +271,33 @@ size_t batch_smem_bytes() {
 }
 
 template <typename T>
+const void* batch_kernel(bool groups) {
+    return groups ? reinterpret_cast<const void*>(k_batch_loop<T, true>)
+                  : reinterpret_cast<const void*>(k_batch_loop<T, false>);
+}
+
+template <typename T>
 cudaError_t batch_occupancy(int* blocks_per_sm) {
     const size_t smem = batch_smem_bytes<T>();
-    cudaError_t e = cudaFuncSetAttribute(k_batch_loop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_batch_loop<T>, kWarps * 32, smem);
+    *blocks_per_sm = 1 << 20;
+    for (bool g : {false, true}) {
+        int n = 0;
+        cudaError_t e = cudaFuncSetAttribute(batch_kernel<T>(g), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(smem));
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<T>(g), kWarps * 32, smem);
+        if (e != cudaSuccess) return e;
+        *blocks_per_sm = std::min(*blocks_per_sm, n);
+    }
+    return cudaSuccess;
 }
 
 template <typename T>
 cudaError_t launch_batch_loop(const LoopParams<T>& P, int grid, cudaStream_t s) {
     LoopParams<T> copy = P;
     void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_batch_loop<T>), dim3(grid), dim3(kWarps * 32),
-                                       args, batch_smem_bytes<T>(), s);
+    return cudaLaunchCooperativeKernel(batch_kernel<T>(P.groups != 0), dim3(grid), dim3(kWarps * 32), args,
+                                       batch_smem_bytes<T>(), s);
 }
 
 }  // namespace eikg

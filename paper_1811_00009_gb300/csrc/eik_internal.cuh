@@ -78,6 +78,7 @@ struct Ctrl {
     int32_t head[kRing];       // next brick work-list entry to hand out
     int32_t pad_head[28];
     int32_t used[kRing];       // length a ring slot's list had when its restart ended (cleared to -1 next restart)
+    int32_t gused[kRing];      // as used, for the group lists
     int32_t gcount[kRing];     // group (16^3 block) work-list lengths, by ring slot
     int32_t ghead[kRing];      // next group work-list entry to hand out
     int32_t mode;              // block edge of restart k: 8 (one warp per brick) or 16 (one CTA per group)
@@ -172,7 +173,8 @@ struct LoopParams {
     int32_t GX, GY, GZ;        // groups of 2x2x2 bricks per axis
     int32_t groups;            // non-zero: keep the group work lists (16^3 restarts possible)
     int32_t* qgroup;           // kRing x ngroups, as queued
-    int32_t* glist[kRing];     // group work lists by ring slot
+    int32_t* glist[kRing];     // group work lists by ring slot; unused entries are -1
+    int32_t* gdone;            // per group: last restart whose march of it finished (null: the schedule may mix block edges)
     int32_t early;             // non-zero: waiting warps may march the next restart's bricks early
     int32_t own_bz0, own_bz1;  // brick planes (z) this launch owns: bricks outside are ghosts of a grid
                                // sharded across GPUs (their faces are imported; never put on a work list)

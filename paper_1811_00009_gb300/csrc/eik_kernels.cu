@@ -179,6 +179,7 @@ __device__ void restart_end(const LoopParams<T>& P, int lane, float* scratch) {
     C->r_rmin_bits = 0x7f800000u;
     C->r_rmax_bits = 0u;
     C->used[s] = __ldcg(&C->count[s]);
+    C->gused[s] = __ldcg(&C->gcount[s]);
     C->count[s] = 0;
     C->head[s] = 0;
     C->gcount[s] = 0;
@@ -236,6 +237,7 @@ __device__ void load_restart(const LoopParams<T>& P, CtaLoop& S) {
     const unsigned gen = __ldcg(&C->bar_gen);
     const double bound = __ldcg(&C->bound), bprev = __ldcg(&C->bound_prev);
     const int n = __ldcg(&C->count[k % kRing]), used = __ldcg(&C->used[(k + kRing - 1) % kRing]);
+    const int gused = __ldcg(&C->gused[(k + kRing - 1) % kRing]);
     double ns;
     int nm;
     next_restart_of(P, C, &ns, &nm);
@@ -244,6 +246,7 @@ __device__ void load_restart(const LoopParams<T>& P, CtaLoop& S) {
     S.mode = mode;
     S.n = mode == 8 ? n : 0;
     S.used = P.early ? used : 0;
+    S.gused = gused;
     S.gen = gen;
     S.early = (P.early && mode == 8 && nm == 8) ? 1 : 0;
     S.bound = bound;
@@ -256,7 +259,86 @@ __device__ void load_restart(const LoopParams<T>& P, CtaLoop& S) {
     S.grow_next = S.next_bound < P.width;
 }
 
+// The restart loop of a fixed schedule with 16^3 blocks, one CTA per group of 2x2x2
+// bricks: a restart's list and, once the CTA has arrived at the barrier, the groups
+// of restart k+1 whose neighbourhood has finished restart k.  (A kernel of its own:
+// with this loop in k_restart_loop its 8^3 marches ran 2 % slower.)  Without early
+// groups a restart of 256^3 lasted as long as its longest march, 77 us against 28 us
+// on average; with them 55 us.
 template <typename T>
+__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_group_loop(const __grid_constant__ LoopParams<T> P) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_item[2];
+    __shared__ CtaLoop S;
+    __shared__ MarchAcc s_acc[kWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Ctrl* C = P.ctrl;
+    MarchAcc& A = s_acc[warp];
+    if (threadIdx.x == 0) {
+        S.arrived = 0;
+        S.claim = 0ull;
+        reset_acc(S.acc);
+        load_restart(P, S);
+        S.rel = S.gen;
+    }
+    if (lane == 0) reset_acc(A);
+    __syncthreads();
+    const Geo G{P.BX, P.BY, P.BZ, 0, P.GX, P.GY, 0, 2u, P.div_x, P.div_xy};
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long t0 = globaltimer();
+        C->t_begin = t0;
+        C->t_restart = t0;
+    }
+    for (;;) {
+        const int k = S.k, s = k % kRing;
+        const unsigned gen = S.gen;
+        // (the waiting CTA's state may become the next restart's)
+        const T bound = pick<T>(S.bound, S.bound_f), bprev = pick<T>(S.bprev, S.bprev_f);
+        const T next = pick<T>(S.next_bound, S.next_f);
+        const bool grow = S.grow != 0, grow_next = S.grow_next != 0;
+        clear_used_slot(P.glist[(k + kRing - 1) % kRing], S.gused);
+        const int n = __ldcg(&C->gcount[s]);
+        bool waiting = false;
+        for (;;) {
+            __syncthreads();
+            int g = -1;
+            if (!waiting) {
+                if (threadIdx.x == 0) {
+                    const bool mine = static_cast<int>(S.claim >> 32) == k;      // claimed while waiting
+                    const int i = mine ? static_cast<int>(S.claim) : atomicAdd(&C->ghead[s], 1);
+                    if (mine) S.claim = 0ull;
+                    s_item[0] = i < n ? __ldcg(P.glist[s] + i) : -1;
+                }
+                __syncthreads();
+                g = s_item[0];
+                if (g < 0) {
+                    if (barrier_arrive(C, S, A, true, lane)) {
+                        restart_end<T>(P, lane, reinterpret_cast<float*>(smem_raw) + warp * 2048);
+                        barrier_release(C, lane, gen);
+                    }
+                    waiting = true;
+                    continue;
+                }
+            } else {
+                const int st = wait_or_group(P, S, k, gen, s_item, &g, [&]() { load_restart(P, S); });
+                if (st == 2) return;
+                if (st == 1) break;
+            }
+            const int gz = g / (P.GX * P.GY), gy = (g / P.GX) % P.GY, gx = g % P.GX, kk = waiting ? k + 1 : k;
+            march16<T>(P, G, A, gx, gy, gz, kk, waiting ? bound : bprev, waiting ? next : bound,
+                       waiting ? grow_next : grow, pick<T>(P.window, P.window_f));
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) st_release(P.gdone + g, kk);
+        }
+        if (S.done) return;
+    }
+}
+
+// The restart loop of 8^3 blocks; MIXED: of a schedule whose restarts may also
+// have 16^3 blocks (learned, random).  (A template: with march16 in the loop the
+// compiler has fewer registers for march8.)
+template <typename T, bool MIXED>
 __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart_loop(const __grid_constant__ LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
@@ -283,12 +365,11 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
     if (lane == 0) reset_acc(A);
     init_queue_smem(SQ[warp], lane);
     __syncthreads();
-    // Work lists the marches fill: the brick list, and for fixed 16^3 blocks
-    // the group list too.  Under a learned or random schedule a 16^3 restart
-    // builds its group list from its brick list when it starts (such restarts
-    // are rare, and every enqueue would otherwise pay for the group list).
-    const Geo G{P.BX, P.BY, P.BZ, 0, P.GX, P.GY, 0, (P.groups && P.sched == 0) ? 3u : 1u,
-                P.div_x, P.div_xy};
+    // The marches fill the brick list.  A 16^3 restart of a learned or random
+    // schedule builds its group list from its brick list when it starts (such
+    // restarts are rare, and every enqueue would otherwise pay for the group list;
+    // a fixed schedule with 16^3 blocks runs in k_group_loop).
+    const Geo G{P.BX, P.BY, P.BZ, 0, P.GX, P.GY, 0, 1u, P.div_x, P.div_xy};
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned long long t0 = globaltimer();
         C->t_begin = t0;
@@ -300,10 +381,9 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart
         const int s = k % kRing;
         const unsigned gen = S.gen;
         keep_restart(L, S, lane);
-        clear_used_slot(P, k, S.used);
-        if (S.mode == 16) {
-            const bool ok = (G.lists & 2u) ||
-                            groups_from_bricks(C, P.list[s], P.qgroup + static_cast<int64_t>(s) * P.ngroups,
+        clear_used_slot(P.list[(k + kRing - 1) % kRing], S.used);
+        if (MIXED && S.mode == 16) {
+            const bool ok = groups_from_bricks(C, P.list[s], P.qgroup + static_cast<int64_t>(s) * P.ngroups,
                                                P.glist[s], s, k, P.BX, P.BY, P.GX, P.GY, P.wait_limit);
             if (!cta_go(C, ok, lane, &s_arrived)) return;
             // one CTA per group of 2x2x2 bricks
@@ -690,21 +770,35 @@ size_t loop_smem_bytes() {
     return std::max(sizeof(GroupSmem<T>), sizeof(QueueSmem<T>) * kWarps);
 }
 
+// Fixed schedules: 8^3 blocks (0) and 16^3 blocks (1); schedules that mix them (2).
+template <typename T>
+const void* loop_kernel(int kind) {
+    return kind == 1   ? reinterpret_cast<const void*>(k_group_loop<T>)
+           : kind == 2 ? reinterpret_cast<const void*>(k_restart_loop<T, true>)
+                       : reinterpret_cast<const void*>(k_restart_loop<T, false>);
+}
+
 template <typename T>
 cudaError_t loop_occupancy(int* blocks_per_sm) {
     const size_t smem = loop_smem_bytes<T>();
-    cudaError_t e = cudaFuncSetAttribute(k_restart_loop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_restart_loop<T>, kWarps * 32, smem);
+    *blocks_per_sm = 1 << 20;
+    for (int kind = 0; kind < 3; ++kind) {
+        const void* f = loop_kernel<T>(kind);
+        int n = 0;
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kWarps * 32, smem);
+        if (e != cudaSuccess) return e;
+        *blocks_per_sm = std::min(*blocks_per_sm, n);
+    }
+    return cudaSuccess;
 }
 
 template <typename T>
 cudaError_t launch_restart_loop(const LoopParams<T>& P, int grid, cudaStream_t s) {
     LoopParams<T> copy = P;
     void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_restart_loop<T>), dim3(grid),
-                                       dim3(kWarps * 32), args, loop_smem_bytes<T>(), s);
+    return cudaLaunchCooperativeKernel(loop_kernel<T>(P.gdone != nullptr ? 1 : P.groups ? 2 : 0), dim3(grid), dim3(kWarps * 32), args,
+                                       loop_smem_bytes<T>(), s);
 }
 
 #define EIKG_INSTANTIATE(T)                                                                                     \

@@ -469,9 +469,7 @@ __device__ __forceinline__ void enqueue_next(const LoopParams<T>& P, const Geo& 
 // coalesced.  The slot is next written in restart k+1 (by early marches of
 // restart k+2 while waiting at its barrier) at the earliest, after every warp has
 // arrived at the barrier of restart k and so has finished its share.
-template <typename T>
-__device__ __forceinline__ void clear_used_slot(const LoopParams<T>& P, int k, int used) {
-    int32_t* list = P.list[(k + kRing - 1) % kRing];
+__device__ __forceinline__ void clear_used_slot(int32_t* list, int used) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < used; i += gridDim.x * blockDim.x) list[i] = -1;
 }
 
@@ -519,7 +517,7 @@ struct CtaLoop {
     int done;
     int mode;                  // block edge
     int n;                     // length of the brick list
-    int used;                  // length of the list to clear
+    int used, gused;           // lengths of the lists to clear
     int early;                 // early work allowed while waiting at this restart's barrier
     int grow, grow_next;       // bound, next_bound below width_band (pending nodes re-activate the block)
     double bound, bprev, next_bound;
@@ -763,6 +761,75 @@ __device__ int wait_or_work(const LoopParams<T>& P, CtaLoop& S, int k, unsigned 
         give_up(C, lane);
         return 2;
     }
+    return st;
+}
+
+// The same for a CTA that marches 16^3 blocks, as a whole: its first thread polls,
+// claims (open claim: S.claim) and waits until the group and each of its six
+// neighbours on restart k's list have finished that march.  1: released, 2:
+// leave, 3: *g is a group of restart k+1.
+template <typename T, typename Load>
+__device__ int wait_or_group(const LoopParams<T>& P, CtaLoop& S, int k, unsigned gen, int* s_answer, int* g, Load load) {
+    Ctrl* C = P.ctrl;
+    const int s = k % kRing, s1 = (k + 1) % kRing;
+    if (threadIdx.x == 0) {
+        int st = 0;
+        int32_t x = -1;
+        unsigned nap = 32;
+        for (long long it = 0; st == 0; ++it) {
+            if (ld_acquire(&C->bar_gen) != gen) {
+                load();
+                S.rel = gen + 1;
+                st = 1;
+                break;
+            }
+            if (__ldcg(&C->status) & kStWaitTimeout) {
+                st = 2;
+                break;
+            }
+            const unsigned long long mine = static_cast<unsigned long long>(k + 1) << 32;
+            const int c = (S.claim >> 32) == (mine >> 32) ? static_cast<int>(S.claim) : atomicAdd(&C->ghead[s1], 1);
+            const bool have = c < __ldcg(&C->gcount[s1]);
+            S.claim = have ? 0ull : mine | static_cast<unsigned>(c);
+            if (have) {
+                st = 3;
+                x = ld_acquire(P.glist[s1] + c);
+                for (long long w = 0; x < 0 && w < P.wait_limit; ++w) {
+                    __nanosleep(32);
+                    x = ld_acquire(P.glist[s1] + c);
+                }
+                const int gx = x % P.GX, gy = (x / P.GX) % P.GY, gz = x / (P.GX * P.GY);
+                const int32_t near[7] = {x, gx > 0 ? x - 1 : -1, gx < P.GX - 1 ? x + 1 : -1, gy > 0 ? x - P.GX : -1,
+                                         gy < P.GY - 1 ? x + P.GX : -1, gz > 0 ? x - P.GX * P.GY : -1,
+                                         gz < P.GZ - 1 ? x + P.GX * P.GY : -1};
+                long long w = x < 0 ? P.wait_limit + 1 : 0;
+                for (int j = 0; j < 7 && w <= P.wait_limit; ++j) {
+                    if (near[j] < 0 || __ldcg(P.qgroup + static_cast<int64_t>(s) * P.ngroups + near[j]) != k) continue;
+                    unsigned d = 64;
+                    for (w = 0; ld_acquire(P.gdone + near[j]) < k && w <= P.wait_limit; ++w) {
+                        __nanosleep(d);
+                        if (d < 512) d <<= 1;
+                    }
+                }
+                if (w > P.wait_limit) st = 4;
+                break;
+            }
+            if (it > P.wait_limit) st = 4;
+            __nanosleep(nap);
+            if (nap < 512) nap <<= 1;
+        }
+        if (st == 4) {
+            atomicOr(&C->status, kStWaitTimeout);
+            __threadfence();
+            st = 2;
+        }
+        s_answer[0] = st;
+        s_answer[1] = x;
+    }
+    __syncthreads();
+    const int st = s_answer[0];
+    *g = s_answer[1];
+    __syncthreads();                           // (read before the first thread answers again)
     return st;
 }
 

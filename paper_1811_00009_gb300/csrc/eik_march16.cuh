@@ -7,12 +7,11 @@
 // solve are kept in two lists: a wave solves the nodes of one, 32 per warp at a
 // time, and queues the neighbours that an accepted node can lower into the other.
 //
-// The warps of a wave run without barriers.  A node is in a list at most once, so
-// one warp alone writes its value.  A neighbour's value may be read before or
-// after that neighbour's own solve of this wave; either is an upper bound of what
-// it ends with, and a reader that was too early is queued again: a warp clears a
-// node's queue mark before it reads the neighbours, and sets marks only after it
-// has written the value, so a mark found set belongs to a reader still to come.
+// A node is in a list at most once, so one thread alone writes its value in a wave.
+// A neighbour's value may be read before or after that neighbour's own solve of
+// the wave; either is an upper bound of what it ends with, and as the wave starts
+// with clearing its nodes' queue marks, a neighbour that is lowered queues them
+// again for the next.
 //
 // What bounds it: the chain of waves (two of its three latencies are shared-memory
 // round trips) and, with all SMs busy, issue slots.  The march this replaces gave
@@ -69,11 +68,10 @@ __device__ __forceinline__ void append(uint16_t* list, int* count, bool in, int 
     if (in) list[base + __popc(m & ((1u << lane) - 1u))] = static_cast<uint16_t>(h);
 }
 
-// Group (gx, gy, gz) of grid G at restart k; every thread of the CTA.  Out of line:
-// the loop around it keeps its registers for march8.
+// Group (gx, gy, gz) of grid G at restart k; every thread of the CTA.
 template <typename T>
-__device__ __noinline__ void march16(const LoopParams<T>& P, const Geo& G, MarchAcc& A, int gx, int gy, int gz, int k,
-                                     T bprev, T bound, bool grow, T window) {
+__device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, MarchAcc& A, int gx, int gy, int gz, int k,
+                                        T bprev, T bound, bool grow, T window) {
     static_assert(kWarps == 8, "a warp per brick of the group");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GroupSmem<T>& S = *reinterpret_cast<GroupSmem<T>*>(smem_raw);
@@ -260,23 +258,27 @@ __device__ __noinline__ void march16(const LoopParams<T>& P, const Geo& G, March
             for (int s = 0; s < 2; ++s)
 #pragma unroll
                 for (int x = 0; x < 8; ++x) {
-                    const int h = hbase + kUp * s + x;
-                    const SB v = sbits(S.psi[h]);
-                    if (v > tk) smin = min(smin, v);
-                    const int w0 = ld_word(sign_word(S.rq + h));
-                    const bool in = v <= tk && (w0 >= 0 || !(vabs(S.rq[h]) < INF));
-                    if (in) st_word(sign_word(S.rq + h), w0 | static_cast<int>(0x80000000u));
-                    C |= (in ? 1u : 0u) << (8 * s + x);
+                    const SB v = sbits(S.psi[hbase + kUp * s + x]);
+                    if (v <= tk) C |= 1u << (8 * s + x);
+                    else smin = min(smin, v);
                 }
-            const int cnt = __popc(C);
-            int incl = cnt;
+            if (__any_sync(kFull, C != 0u)) {                    // (a brick the front is not in has none)
+                const uint32_t rw = sign_word(S.rq + hbase);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const int total = __shfl_sync(kFull, incl, 31);
-            if (total > 0) {
+                for (int j = 0; j < 16; ++j) {
+                    const int h = (j >> 3) * kUp + (j & 7);
+                    const int w0 = ld_word(rw + h * static_cast<int>(sizeof(T)));
+                    if (w0 < 0 && vabs(S.rq[hbase + h]) < INF) C &= ~(1u << j);
+                    if ((C >> j) & 1u) st_word(rw + h * static_cast<int>(sizeof(T)), w0 | static_cast<int>(0x80000000u));
+                }
+                const int cnt = __popc(C);
+                int incl = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const int total = __shfl_sync(kFull, incl, 31);
                 int base = 0;
                 if (lane == 0) base = atomicAdd(&S.count[wave % 3], total);
                 uint16_t* at = S.list[wave & 1] + __shfl_sync(kFull, base, 0) + (incl - cnt);
@@ -297,16 +299,21 @@ __device__ __noinline__ void march16(const LoopParams<T>& P, const Geo& G, March
             const uint16_t* from = S.list[wave & 1];
             uint16_t* to = S.list[(wave + 1) & 1];
             int* fill = &S.count[(wave + 1) % 3];
-            for (int base = 32 * warp; base < n; base += 32 * kWarps) {
-                const bool val = base + lane < n;
+            // the listed nodes may be queued again from here on
+            for (int i = threadIdx.x; i < n; i += 32 * kWarps) {
+                T* p = S.rq + from[i];
+                const T r = vabs(*p);
+                if (r < INF) *p = r;
+            }
+            __syncthreads();
+            for (int base = 0; base < n; base += 32 * kWarps) {
+                const bool val = base + static_cast<int>(threadIdx.x) < n;
                 n_solve += val ? 1u : 0u;
-                const int hq = val ? from[base + lane] : h16(0, 0, 0);
+                const int hq = val ? from[base + threadIdx.x] : h16(0, 0, 0);
                 T* ps = S.psi + hq;
+                volatile const T* pv = ps;
                 const T r = vabs(S.rq[hq]);
                 const bool live = val && r < INF;                // (a fixed node only passes its value on)
-                if (live) *const_cast<volatile T*>(&S.rq[hq]) = r;   // may be queued again, from here on
-                __threadfence_block();
-                volatile const T* pv = ps;
                 const T cur = pv[0], c = vabs(cur);
                 const T nv[6] = {pv[-1], pv[1], pv[-kH16], pv[kH16], pv[-kUp], pv[kUp]};
                 const T mx = axis_min(nv[0], nv[1]), my = axis_min(nv[2], nv[3]), mz = axis_min(nv[4], nv[5]);
@@ -321,14 +328,27 @@ __device__ __noinline__ void march16(const LoopParams<T>& P, const Geo& G, March
                 if (imp && !prop) smin = min(smin, sbits(-v));
                 n_upd += imp ? 1u : 0u;
                 n_acc += prop ? 1u : 0u;
-                __threadfence_block();
+                // queue the neighbours above the accepted value, each once, by marks as in
+                // march8; marks are negative, so a warp that is a round ahead leaves them be
                 constexpr int off[6] = {-1, 1, -kH16, kH16, -kUp, kUp};
+                const int mark = (sizeof(T) == 4 ? static_cast<int>(0xFFC00000u) : static_cast<int>(0xFFF80000u)) |
+                                 static_cast<int>(threadIdx.x);
                 const uint32_t rw = sign_word(S.rq + hq);
+                int nw[6];
                 bool win[6];
+#pragma unroll
+                for (int d = 0; d < 6; ++d) {
+                    nw[d] = ld_word(rw + off[d] * static_cast<int>(sizeof(T)));
+                    win[d] = prop && vlt(v, vabs(nv[d])) && nw[d] >= 0;
+                }
+#pragma unroll
+                for (int d = 0; d < 6; ++d)
+                    if (win[d]) st_word(rw + off[d] * static_cast<int>(sizeof(T)), mark);
+                __syncthreads();
                 unsigned cnt = 0;
 #pragma unroll
                 for (int d = 0; d < 6; ++d) {
-                    win[d] = claim_sign(rw + off[d] * static_cast<int>(sizeof(T)), prop && vlt(v, vabs(nv[d])));
+                    win[d] = win[d] && ld_word(rw + off[d] * static_cast<int>(sizeof(T))) == mark;
                     cnt += win[d] ? 1u : 0u;
                 }
                 const unsigned c0 = __ballot_sync(kFull, cnt & 1u), c1 = __ballot_sync(kFull, cnt & 2u);
@@ -340,7 +360,10 @@ __device__ __noinline__ void march16(const LoopParams<T>& P, const Geo& G, March
                     at = __shfl_sync(kFull, at, 0) + __popc(c0 & lt) + 2 * __popc(c1 & lt) + 4 * __popc(c2 & lt);
 #pragma unroll
                     for (int d = 0; d < 6; ++d)
-                        if (win[d]) to[at++] = static_cast<uint16_t>(hq + off[d]);
+                        if (win[d]) {
+                            to[at++] = static_cast<uint16_t>(hq + off[d]);
+                            st_word(rw + off[d] * static_cast<int>(sizeof(T)), nw[d] | static_cast<int>(0x80000000u));
+                        }
                 }
             }
             __syncthreads();

@@ -78,6 +78,7 @@ struct eik_ctx {
     int64_t ngroups = 0;
     int32_t* qgroup = nullptr;     // kRing x ngroups
     int32_t* glists = nullptr;     // kRing x ngroups
+    int32_t* gdone = nullptr;      // per group
     eikg::Ctrl* ctrl = nullptr;
     // Mapped pinned host memory that kernels write directly, so that the host
     // reads small results after a stream synchronisation without a
@@ -163,7 +164,7 @@ cudaError_t dalloc(P** p, size_t bytes) {
 }
 
 void free_all(eik_ctx* c) {
-    void* ptrs[] = {c->rr,    c->slot,  c->ups,   c->stamp,   c->queued, c->lists, c->done, c->qgroup, c->glists,
+    void* ptrs[] = {c->rr,    c->slot,  c->ups,   c->stamp,   c->queued, c->lists, c->done, c->qgroup, c->glists, c->gdone,
                     c->ctrl,  c->log, c->scratch, c->fstage, c->d_mlp};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -323,6 +324,7 @@ eik_status eik_create(eik_ctx** out, const int32_t dims[3], double h, const void
         {reinterpret_cast<void**>(&c->done), nb * sizeof(int32_t)},
         {reinterpret_cast<void**>(&c->qgroup), eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t)},
         {reinterpret_cast<void**>(&c->glists), eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t)},
+        {reinterpret_cast<void**>(&c->gdone), static_cast<size_t>(c->ngroups) * sizeof(int32_t)},
         {reinterpret_cast<void**>(&c->ctrl), sizeof(eikg::Ctrl)},
     };
     for (auto& a : allocs) {
@@ -586,6 +588,7 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
     if (groups) {
         EIK_CK(c, cudaMemsetAsync(c->qgroup, 0xFF, eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
         EIK_CK(c, cudaMemsetAsync(c->glists, 0xFF, eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
+        EIK_CK(c, cudaMemsetAsync(c->gdone, 0, static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
     }
     if (nfix > 0)
         EIK_CK(c, eikg::launch_init_sources<T>(nfix, c->d_fix_b, c->d_fix_p, d_fv, static_cast<int>(sb.size()), d_sb,
@@ -641,6 +644,8 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
             L.glist[r] = c->glists + r * c->ngroups;
         }
         L.early = 1;
+        // (a fixed schedule of 16^3 blocks: a kernel of its own, which keeps the group list a restart ahead)
+        L.gdone = (groups && P.schedule == EIK_SCHED_FIXED) ? c->gdone : nullptr;
         L.GX = c->GX;
         L.GY = c->GY;
         L.GZ = c->GZ;

@@ -1,4 +1,4 @@
-"""The queue march of the 8^3 blocks (eik_march8.cuh) where it can go wrong: rough speeds (many stages in a
+"""The queue marches of the 8^3 and 16^3 blocks (eik_march8.cuh, eik_march16.cuh) where they can go wrong: rough speeds (many stages in a
 march, corrections of accepted values), barriers, sources on block faces, grids of one node to a few blocks with
 ragged edges, and windows and strides from one node a stage to the whole block at once.
 
@@ -53,12 +53,14 @@ def test_rough_speeds_and_barriers(eik, orc, dims, precision):
         S.add_sources(src)
         for v in VARIANTS:
             kw = dict(v)
-            S.solve(kw.pop("stride") * h, block_dim=8, **kw)
-            psi = S.result()
-            assert np.array_equal(np.isfinite(psi), fin), v
-            if precision == "fp64":
-                assert np.all(np.abs(psi[fin] - ref[fin]) <= 1e-12 * ref[fin]), v
-            else:
-                assert np.max(np.abs(psi[fin].astype(np.float64) - ref[fin])) <= 1e-5 * ref[fin].max(), v
-            base = psi.copy() if base is None else base
-            assert np.array_equal(psi, base), v
+            stride = kw.pop("stride") * h
+            for edge in (8, 16):
+                S.solve(stride, block_dim=edge, **kw)
+                psi = S.result()
+                assert np.array_equal(np.isfinite(psi), fin), (v, edge)
+                if precision == "fp64":
+                    assert np.all(np.abs(psi[fin] - ref[fin]) <= 1e-12 * ref[fin]), (v, edge)
+                else:
+                    assert np.max(np.abs(psi[fin].astype(np.float64) - ref[fin])) <= 1e-5 * ref[fin].max(), (v, edge)
+                base = psi.copy() if base is None else base
+                assert np.array_equal(psi, base), (v, edge)
