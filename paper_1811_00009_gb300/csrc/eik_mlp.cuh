@@ -29,30 +29,4 @@ __host__ __device__ inline double action_stride_h(int a) {
 }
 __host__ __device__ inline int action_block(int a) { return a < 8 ? 8 : 16; }
 
-// One sample, one thread: outputs y and (optionally) the hidden activations.
-__device__ inline void mlp_forward_one(const float* __restrict__ w, const float* x, float* y, float* h1o, float* h2o) {
-    float h1[kHid], h2[kHid];
-#pragma unroll 4
-    for (int i = 0; i < kHid; ++i) {
-        float s = w[kOffB1 + i];
-        for (int j = 0; j < kIn; ++j) s += w[kOffW1 + i * kIn + j] * x[j];
-        h1[i] = tanhf(s);
-    }
-#pragma unroll 4
-    for (int i = 0; i < kHid; ++i) {
-        float s = w[kOffB2 + i];
-        for (int j = 0; j < kHid; ++j) s += w[kOffW2 + i * kHid + j] * h1[j];
-        h2[i] = tanhf(s);
-    }
-    for (int a = 0; a < kAct; ++a) {
-        float s = w[kOffB3 + a];
-        for (int j = 0; j < kHid; ++j) s += w[kOffW3 + a * kHid + j] * h2[j];
-        y[a] = s;
-    }
-    if (h1o)
-        for (int i = 0; i < kHid; ++i) h1o[i] = h1[i];
-    if (h2o)
-        for (int i = 0; i < kHid; ++i) h2o[i] = h2[i];
-}
-
 }  // namespace eikg
