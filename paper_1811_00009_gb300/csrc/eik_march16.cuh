@@ -194,7 +194,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
             const T v = row[8 * s + x];
-            const T t = (v < INF && (v > bprev || ((again >> (8 * s + x)) & 1u))) ? -v : v;
+            const T t = ((again >> (8 * s + x)) & 1u) ? -v : band_value(v, bprev);
             S.psi[hbase + kUp * s + x] = t;
             smin = min(smin, sbits(t));
         }
@@ -203,8 +203,8 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
     for (int f = 0; f < 6; ++f) {
         const T v = fv[f];
         const unsigned um = __shfl_sync(kFull, half ? static_cast<unsigned>(mups >> 32) : static_cast<unsigned>(mups), f);
-        const bool tent = v < INF && (((um >> lane) & 1u) || v > bprev);
-        const bool take = tent && v <= bound;
+        const bool tent = vlt(v, INF) && (((um >> lane) & 1u) || sbits(v) > sbits(bprev));
+        const bool take = tent && sbits(v) <= sbits(bound);
         S.psi[ghost(f)] = tent && !take ? -v : v;
         S.rq[ghost(f)] = -INF;
         if (take) smin = min(smin, sbits(-v));
@@ -268,7 +268,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
                 for (int j = 0; j < 16; ++j) {
                     const int h = (j >> 3) * kUp + (j & 7);
                     const int w0 = ld_word(rw + h * static_cast<int>(sizeof(T)));
-                    if (w0 < 0 && vabs(S.rq[hbase + h]) < INF) C &= ~(1u << j);
+                    if (w0 < 0 && vlt(vabs(S.rq[hbase + h]), INF)) C &= ~(1u << j);
                     if ((C >> j) & 1u) st_word(rw + h * static_cast<int>(sizeof(T)), w0 | static_cast<int>(0x80000000u));
                 }
                 const int cnt = __popc(C);
@@ -303,7 +303,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
             for (int i = threadIdx.x; i < n; i += 32 * kWarps) {
                 T* p = S.rq + from[i];
                 const T r = vabs(*p);
-                if (r < INF) *p = r;
+                if (vlt(r, INF)) *p = r;
             }
             __syncthreads();
             for (int base = 0; base < n; base += 32 * kWarps) {
@@ -313,7 +313,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
                 T* ps = S.psi + hq;
                 volatile const T* pv = ps;
                 const T r = vabs(S.rq[hq]);
-                const bool live = val && r < INF;                // (a fixed node only passes its value on)
+                const bool live = val && vlt(r, INF);            // (a fixed node only passes its value on)
                 const T cur = pv[0], c = vabs(cur);
                 const T nv[6] = {pv[-1], pv[1], pv[-kH16], pv[kH16], pv[-kUp], pv[kUp]};
                 const T mx = axis_min(nv[0], nv[1]), my = axis_min(nv[2], nv[3]), mz = axis_min(nv[4], nv[5]);
@@ -321,7 +321,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
                 sort3(mx, my, mz, a0, a1, a2);
                 const bool go = live && vlt(a0, INF);
                 const T xn = QueueRoot<T>::go(a0, a1, a2, r, go, P.tau_f, n_fb);
-                const bool imp = go && xn < c;
+                const bool imp = go && vlt(xn, c);
                 const T v = imp ? xn : c;
                 const bool prop = val && (imp || sgn(cur)) && !vlt(thr, v);
                 if (imp || prop) *const_cast<volatile T*>(ps) = prop ? v : -v;
