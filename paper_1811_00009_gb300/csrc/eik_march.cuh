@@ -56,7 +56,11 @@ __device__ __forceinline__ double from_bits(unsigned long long u) {
     return __longlong_as_double(static_cast<long long>(u));
 }
 __device__ __forceinline__ float vabs(float v) { return fabsf(v); }
-__device__ __forceinline__ double vabs(double v) { return fabs(v); }
+// (double precision on the bits: the compiler's negation and absolute value of a
+// double are FP64-pipe instructions)
+__device__ __forceinline__ double vabs(double v) { return from_bits(ubits(v) & 0x7fffffffffffffffull); }
+__device__ __forceinline__ float vneg(float v) { return -v; }
+__device__ __forceinline__ double vneg(double v) { return from_bits(ubits(v) ^ 0x8000000000000000ull); }
 // Min, max and order of values that are >= 0 or +inf (every use in the march):
 // single precision on the FP32 units; double precision as integer operations on
 // the bit patterns, which order like such values, keeping them off this part's

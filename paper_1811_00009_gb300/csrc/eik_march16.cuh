@@ -194,7 +194,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
             const T v = row[8 * s + x];
-            const T t = ((again >> (8 * s + x)) & 1u) ? -v : band_value(v, bprev);
+            const T t = ((again >> (8 * s + x)) & 1u) ? vneg(v) : band_value(v, bprev);
             S.psi[hbase + kUp * s + x] = t;
             smin = min(smin, sbits(t));
         }
@@ -205,9 +205,9 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
         const unsigned um = __shfl_sync(kFull, half ? static_cast<unsigned>(mups >> 32) : static_cast<unsigned>(mups), f);
         const bool tent = vlt(v, INF) && (((um >> lane) & 1u) || sbits(v) > sbits(bprev));
         const bool take = tent && sbits(v) <= sbits(bound);
-        S.psi[ghost(f)] = tent && !take ? -v : v;
+        S.psi[ghost(f)] = tent && !take ? vneg(v) : v;
         S.rq[ghost(f)] = -INF;
-        if (take) smin = min(smin, sbits(-v));
+        if (take) smin = min(smin, sbits(vneg(v)));
         fire |= (take ? 1u : 0u) << f;
     }
     const T rmin_w = warp_min_nn(from_bits(rlo)), rmax_w = warp_max(from_bits(static_cast<UB>(rhi)));
@@ -223,7 +223,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
     };
     {
         const T m = warp_min_sb(smin);
-        if (lane == 0 && m < INF) atomicMin(&S.mn[0], sbits(-m));
+        if (lane == 0 && m < INF) atomicMin(&S.mn[0], sbits(vneg(m)));
     }
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
@@ -247,7 +247,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
             break;
         }
         const T thr = vmin(mn + w, bound);
-        const SB tk = sbits(-thr);
+        const SB tk = sbits(vneg(thr));
         // ---- tentative nodes up to thr -> the list, and the smallest above it.  (A
         // node already listed, next to an accepted ghost node, is not listed again; a
         // fixed node is never marked and only passes its value on.)
@@ -324,8 +324,8 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
                 const bool imp = go && vlt(xn, c);
                 const T v = imp ? xn : c;
                 const bool prop = val && (imp || sgn(cur)) && !vlt(thr, v);
-                if (imp || prop) *const_cast<volatile T*>(ps) = prop ? v : -v;
-                if (imp && !prop) smin = min(smin, sbits(-v));
+                if (imp || prop) *const_cast<volatile T*>(ps) = prop ? v : vneg(v);
+                if (imp && !prop) smin = min(smin, sbits(vneg(v)));
                 n_upd += imp ? 1u : 0u;
                 n_acc += prop ? 1u : 0u;
                 // queue the neighbours above the accepted value, each once, by marks as in
@@ -372,7 +372,7 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
         {
             const T m = warp_min_sb(smin);
             __syncthreads();                                     // (the other parity's slot is clear)
-            if (lane == 0 && m < INF) atomicMin(&S.mn[stages & 1], sbits(-m));
+            if (lane == 0 && m < INF) atomicMin(&S.mn[stages & 1], sbits(vneg(m)));
         }
         __syncthreads();
     }

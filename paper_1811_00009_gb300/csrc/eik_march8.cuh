@@ -62,7 +62,7 @@ struct SBitsOf<double> {
 // so, and keep the double-precision case off the FP64 pipe).
 template <typename T>
 __device__ __forceinline__ T band_value(T v, T bprev) {
-    return vlt(v, Num<T>::inf()) && sbits(v) > sbits(bprev) ? -v : v;
+    return vlt(v, Num<T>::inf()) && sbits(v) > sbits(bprev) ? vneg(v) : v;
 }
 
 // 32-bit accesses to the words that hold the signs of shared values.
@@ -277,16 +277,18 @@ __device__ __forceinline__ double root_fast(double a, double b, double c, double
     const bool ok = static_cast<unsigned>(sh - 2) <= 42u && Er >= 1 && Ea < 2046;
     const int s = ok ? sh : 2;
     const U A = mantissa(a), R = mantissa(r);
-    // (v - a) in units V; not admitted anyhow, if above h/F: then far above
+    // (v - a) in units V; a value above a + h/F is not admitted: beyond any T
     auto above_a = [&](double v) -> U {
         const int k = (__double2hiint(v) >> 20) - Ea;
         const U d = (k == 1 ? mantissa(v) << 1 : mantissa(v)) - A;
-        return static_cast<unsigned>(k) <= 1u && d <= (R >> s) ? d << s : U(1) << 62;
+        return static_cast<unsigned>(k) <= 1u && d <= (R >> s) ? d << s : (U(1) << 54) - 1;
     };
     const U Db = above_a(b), Dc = above_a(c);
-    // estimate in single precision, in units 2^52 V
-    const float rf = static_cast<float>(R) * 0x1p-52f;
-    const float df = fminf(static_cast<float>(Db) * 0x1p-52f, rf), ef = fminf(static_cast<float>(Dc) * 0x1p-52f, rf);
+    // estimate of T = x - a in single precision, in units 2^52 V
+    const unsigned r31 = static_cast<unsigned>(R >> 22), db = static_cast<unsigned>(Db >> 22);
+    const unsigned dc = static_cast<unsigned>(Dc >> 22);
+    const float rf = static_cast<float>(r31) * 0x1p-30f;
+    const float df = fminf(static_cast<float>(db) * 0x1p-30f, rf), ef = fminf(static_cast<float>(dc) * 0x1p-30f, rf);
     const float rf2 = rf * rf, gf = ef - df;
     const float q1 = __fmaf_rn(-df, df, rf2), q2 = rf2 - __fmaf_rn(gf, gf, ef * ef);
     const bool p1 = q1 > 0.0f, p2 = q2 > 0.0f;
@@ -295,15 +297,21 @@ __device__ __forceinline__ double root_fast(double a, double b, double c, double
     float sum = p1 ? df : 0.0f;
     sum = p2 ? sum + ef : sum;
     const float inv = p2 ? (1.0f / 3.0f) : (p1 ? 0.5f : 1.0f);
-    U T = static_cast<U>(__fmaf_rn(D, rs, sum) * inv * 0x1p52f);       // x - a
-    // two Newton steps: (r^2 - G) / (2 sqrt(D)), the squares' bits from 2^44 up
-    const U R2 = __umul64hi(R << 10, R << 10);
-    const float step = rs * 0x1p-9f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    const unsigned t = static_cast<unsigned>(__fmaf_rn(D, rs, sum) * inv * 0x1p30f);
+    // two Newton steps, (r^2 - G) / (2 sqrt(D)): the first on 31-bit values (from
+    // 2^-21 to 2^-31 of T), the second on the squares' bits from 2^44 up (below a V)
+    U T;
+    {
+        const unsigned tb = t > db ? t - db : 0u, tc = t > dc ? t - dc : 0u;
+        const U G = static_cast<U>(t) * t + static_cast<U>(tb) * tb + static_cast<U>(tc) * tc;
+        const int rho = static_cast<int>(static_cast<long long>(static_cast<U>(r31) * r31 - G) >> 12);
+        T = (static_cast<U>(t) << 22) + (static_cast<long long>(__float2int_rn(static_cast<float>(rho) * (rs * 0x1p-5f))) << 8);
+    }
+    {
         const U tb = T > Db ? (T - Db) << 10 : 0ull, tc = T > Dc ? (T - Dc) << 10 : 0ull;
         const U G = __umul64hi(T << 10, T << 10) + __umul64hi(tb, tb) + __umul64hi(tc, tc);
-        T += __float2ll_rn(static_cast<float>(static_cast<long long>(R2 - G)) * step);
+        const int rho = static_cast<int>(static_cast<long long>(__umul64hi(R << 10, R << 10) - G) >> 6);
+        T += static_cast<long long>(__float2int_rn(static_cast<float>(rho) * (rs * 0x1p-3f)));
     }
     // the double at or below a + T (mantissa X in a's last place, in steps of two from 2^53 up), and the midpoint above it
     U X = A + (T >> s);
@@ -456,8 +464,8 @@ __device__ void march8(const LoopParams<T>& P, const Geo& G, QueueSmem<T>& S, Ma
             const unsigned um = __shfl_sync(kFull, static_cast<unsigned>(mups >> (32 * e)), f);
             const bool tent = vlt(v, INF) && (((um >> lane) & 1u) || sbits(v) > sbits(bprev));
             const bool take = tent && sbits(v) <= sbits(bound);
-            S.psi[ghost(f, e)] = tent && !take ? -v : v;
-            if (take) smin = min(smin, sbits(-v));
+            S.psi[ghost(f, e)] = tent && !take ? vneg(v) : v;
+            if (take) smin = min(smin, sbits(vneg(v)));
             fire |= (take ? 1u : 0u) << (2 * f + e);
         }
     unsigned n_acc = __popc(fire), n_upd = 0u, n_solve = 0u;   // accepted, lowered (per lane), solved (every lane)
@@ -506,7 +514,7 @@ __device__ void march8(const LoopParams<T>& P, const Geo& G, QueueSmem<T>& S, Ma
             break;
         }
         const T thr = vmin(mn + w, bound);
-        const SB tk = sbits(-thr);
+        const SB tk = sbits(vneg(thr));
         // ---- tentative nodes up to thr, and the smallest above it
         SB km = SBitsOf<T>::kMax;
 #pragma unroll
@@ -551,7 +559,7 @@ __device__ void march8(const LoopParams<T>& P, const Geo& G, QueueSmem<T>& S, Ma
             head += n;
             n_solve += n;
             T* ps = S.psi + hq;
-            const T r = -S.rq[hq];
+            const T r = vneg(S.rq[hq]);
             const bool live = val && vlt(r, INF);                // (a fixed node only passes its value on)
             const T cur = ps[0], c = vabs(cur);
             const T nv[6] = {ps[-1], ps[1], ps[-10], ps[10], ps[-100], ps[100]};
@@ -566,8 +574,8 @@ __device__ void march8(const LoopParams<T>& P, const Geo& G, QueueSmem<T>& S, Ma
             const T v = imp ? xn : c;
             const bool prop = val && (imp || sgn(cur)) && !vlt(thr, v);
             __syncwarp();
-            if (imp || prop) ps[0] = prop ? v : -v;
-            if (imp && !prop) smin = min(smin, sbits(-v));
+            if (imp || prop) ps[0] = prop ? v : vneg(v);
+            if (imp && !prop) smin = min(smin, sbits(vneg(v)));
             n_upd += imp ? 1u : 0u;
             n_acc += prop ? 1u : 0u;
             // queue the neighbours above the accepted value, each once: every lane
