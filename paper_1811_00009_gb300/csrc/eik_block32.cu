@@ -3,12 +3,10 @@
 // (Sec. 3.6): a larger block carries the front across more nodes within one
 // restart, so fewer accepted values have to be refreshed when ghost layers
 // change (Sec. 3.5).  A 32^3 tile with a one-node ghost layer (34^3 floats,
-// 157 KB) fits one CTA's shared memory, and so do the bit masks of the march:
-// one 32-bit word per x-row of the block (y + 32 z) holds the row's band
-// (BAND of Sec. 2.1), the nodes accepted in a round, the nodes lowered in the
-// march (Upsilon) and the nodes that are solved at all.  Thread t loads and
-// writes back row t; in the rounds the rows are dealt out diagonally (see
-// round_row) so that a front lying in a plane spreads over all warps.
+// 157 KB) fits one CTA's shared memory, and so do the march's bit masks -- one
+// 32-bit word per x-row of the block (y + 32 z) for its tentative nodes (BAND of
+// Sec. 2.1) -- a byte per node that marks it to be solved, and the list of a wave's
+// nodes.  h/F is read from global memory.  Thread t owns row t's marks and masks.
 //
 // Data layout in HBM (one grid): blocks b = (bz*NBY + by)*NBX + bx of 32^3
 // nodes, node p = (z*32 + y)*32 + x; the ragged last block of each axis is
@@ -29,7 +27,7 @@
 // finished restart k (their done marks), and then reads the same as after the
 // barrier.
 #include "eik_internal.cuh"
-#include "eik_march.cuh"
+#include "eik_march8.cuh"
 
 #include <algorithm>
 #include <cstdint>
@@ -44,7 +42,7 @@ constexpr int kHN = kH * kH * kH;      // halo tile
 constexpr int kCopy = kN + 2 * kE * kE;
 constexpr int kX0 = kN, kX31 = kN + kE * kE;
 constexpr int kT = 1024;               // threads per CTA: one per x-row
-constexpr int kWL = 256;               // per warp: candidates of a solve pass
+constexpr int kCap = 16384;            // nodes the list holds (more stay marked for a later wave)
 
 struct Params {
     int32_t NBX, NBY, NBZ;
@@ -66,17 +64,16 @@ struct Params {
 };
 
 struct __align__(16) Smem {
-    float psi[kHN];                    // tile with ghost layer, index ((z+1)*34 + (y+1))*34 + (x+1)
-    unsigned band[kT];                 // per row: band nodes
-    unsigned acc[2][kT];               // per row: accepted in this round (by round parity)
-    unsigned upd[kT];                  // per row: lowered in this march
+    float psi[kHN];                    // tile with ghost layer, index ((z+1)*34 + (y+1))*34 + (x+1); tentative values negative
+    unsigned band[kT];                 // per row: tentative nodes
     unsigned solv[kT];                 // per row: solved nodes
-    unsigned gband[6][32];             // ghost faces: band nodes (face-local word c, bit a)
-    unsigned gacc[2][6][32];           // ghost faces: accepted in this round
-    unsigned mslot[3];                 // band minimum for round j (float bits) at [j % 3]
-    unsigned wmin;                     // min h/F over the block's solved nodes (float bits)
+    unsigned char mark[kN];            // per node (row*32 + x): to be solved in the next wave
+    unsigned short list[kCap];         // this wave's nodes
     unsigned long long nst[8];         // stamps of the six neighbours and of the block itself
-    unsigned short wl[32][kWL];        // per warp: candidates of a solve pass (node index)
+    int mn[2];                         // smallest tentative value by stage parity (sbits)
+    unsigned wmin;                     // min h/F over the block's solved nodes (float bits)
+    unsigned pend, any;                // pending nodes at the end; the march lowered a value
+    int count[2];                      // length of the list, by wave parity
     int facemask;
 };
 
@@ -110,58 +107,19 @@ __device__ __forceinline__ void enqueue(const Params& P, int k, int32_t x) {
     }
 }
 
-// Row of the rounds' thread mapping: lane l of warp w holds the x-row (y, z) =
-// ((w + l) mod 32, l).  Every plane of constant y or constant z then spreads
-// over all 32 warps (one row each), so a front lying in such a plane gives
-// every warp the same share of a round's work.
-__device__ __forceinline__ int round_row(int warp, int lane) { return lane * kE + ((warp + lane) & 31); }
-
-// Alg. 3 for one candidate node (index idx = row*32 + x) of the tile: per axis
-// the smaller KNOWN neighbour below the node's value (BAND values carry their
-// sign bit and order above every KNOWN bit pattern, as in the 8^3 march), then
-// the upwind root; a lower value makes the node BAND again.
-__device__ __forceinline__ void solve_node(const Params& P, Smem& S, int32_t blk, int idx, float tau, int& fb,
-                                           float& smin, unsigned& nupd) {
-    const float INF = __int_as_float(0x7f800000);
-    const int x = idx & 31, row = idx >> 5;
-    const int hq = ((row >> 5) + 1) * kH * kH + ((row & 31) + 1) * kH + x + 1;
-    const float r = __ldg(P.rr + static_cast<int64_t>(blk) * kN + idx);
-    const float c = fabsf(S.psi[hq]);
-    const unsigned cb = __float_as_uint(c);
-    auto axis = [&](float p, float q) -> float {
-        const unsigned up = __float_as_uint(p), uq = __float_as_uint(q);
-        const unsigned mm = up < uq ? up : uq;
-        return mm < cb ? __uint_as_float(mm) : INF;
-    };
-    const float mx = axis(S.psi[hq - 1], S.psi[hq + 1]);
-    const float my = axis(S.psi[hq - kH], S.psi[hq + kH]);
-    const float mz = axis(S.psi[hq - kH * kH], S.psi[hq + kH * kH]);
-    const float lo = fminf(mx, my), hi = fmaxf(mx, my);
-    const float a0 = fminf(lo, mz), t1 = fmaxf(lo, mz);
-    const float a1 = fminf(hi, t1), a2 = fmaxf(hi, t1);
-    if (a0 < INF) {
-        const float xn = upwind_root_f32(a0, a1, a2, r, tau, fb);
-        if (xn < c) {
-            S.psi[hq] = -xn;                              // tentative again: BAND
-            atomicOr(&S.upd[row], 1u << x);
-            atomicOr(&S.band[row], 1u << x);
-            smin = fminf(smin, xn);
-            ++nupd;
-        }
-    }
-}
+__device__ __forceinline__ void prefetch_l1(const float* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // March_Narrow_Band (Alg. 4 with Algs. 2 and 3) of block blk at restart k, the
-// exchange of Alg. 5 for its ghost layer done first from the neighbours'
-// copies as of the end of restart k-1.  Rounds of windowed ordered acceptance
-// as in the 8^3 march: accept every band node within w of the band minimum
-// (and not above the bound), then re-solve their neighbours.  A round has two
-// CTA barriers: after the acceptance (the accepted rows are read by the
-// neighbouring rows' threads) and after the solves (the next round reads the
-// lowered values and the band minimum, kept by an atomic minimum in shared
-// memory).  Each warp enumerates its words of band nodes and candidates either
-// bit by bit in each lane or row by row across its lanes, whichever takes
-// fewer steps, and solves its own candidates from a list of its own.
+// exchange of Alg. 5 for its ghost layer done first from the neighbours' copies as
+// of the end of restart k-1.  Stages as in the 16^3 march (eik_march16.cuh): a
+// stage settles the tentative nodes up to thr = min(m + 1.5 w, bound), in waves.
+// A wave turns the marks into a list (each thread its row's, cleared as they are
+// read), solves the listed nodes, a thread each, and marks the neighbours an
+// accepted node can lower: a plain store, since a node marked twice is marked once.
+// (Claiming them with shared atomics took 3000 cycles a wave: the SM's atomic unit
+// takes about 30 cycles for a warp's.  A list per warp over rows dealt out
+// diagonally saves the one atomic a warp but leaves the warps unevenly loaded:
+// 13.8 ms against 12.5 on 320^3.)
 __device__ void march32(const Params& P, Smem& S, int32_t blk, int k, float bprev, float bound, bool grow) {
     const float INF = __int_as_float(0x7f800000);
     const unsigned INFB = 0x7f800000u;
@@ -177,250 +135,226 @@ __device__ void march32(const Params& P, Smem& S, int32_t blk, int k, float bpre
     nbr[4] = bz > 0 ? blk - plane : -1;
     nbr[5] = bz < P.NBZ - 1 ? blk + plane : -1;
 
-    // ---- load (thread t holds row t: y = lane, z = warp): the stamps, then the
-    // block's latest copy and h/F of the row
+    // ---- load: the stamps, then the block's latest copy and h/F
     if (t < 7) S.nst[t] = (t == 6) ? __ldcg(P.stamp + blk) : (nbr[t] >= 0 ? __ldcg(P.stamp + nbr[t]) : kUntouched);
     if (t == 0) {
-        S.mslot[0] = S.mslot[1] = S.mslot[2] = INFB;
+        S.mn[0] = S.mn[1] = 0x7fffffff;
         S.wmin = INFB;
+        S.pend = S.any = 0u;
         S.facemask = 0;
+        S.count[0] = S.count[1] = 0;
     }
     __syncthreads();
     const unsigned long long st = S.nst[6];
-    float mn0 = INF, rlo = INF;
-    {
-        const int y = lane, z = warp, rb = hx(0, y, z);
-        const float* rs = P.rr + static_cast<int64_t>(blk) * kN + (z * kE + y) * kE;
-        const float* ps = (st == kUntouched) ? nullptr
-                                              : P.copy + (static_cast<int64_t>(blk) * 2 + stamp_copy(st)) * kCopy +
-                                                    (z * kE + y) * kE;
-        float row[32];
-        unsigned B = 0u, SV = 0u;
+    const int y = lane, z = warp, rb = hx(0, y, z);              // row t
+    const float* rr = P.rr + static_cast<int64_t>(blk) * kN;
+    int smin = 0x7fffffff;
+    float rlo = INF;
+    // the warp's plane z, coalesced: four nodes of row (i, lane / 8) a time, eight lanes a row
+#pragma unroll 4
+    for (int i = 0; i < 8; ++i) {
+        const int row = 4 * i + (lane >> 3), x0 = 4 * (lane & 7);
+        const float4 rv = __ldg(reinterpret_cast<const float4*>(rr + (z * kE + row) * kE + x0));
+        float4 pv = make_float4(INF, INF, INF, INF);
+        if (st != kUntouched)
+            pv = __ldcg(reinterpret_cast<const float4*>(P.copy + (static_cast<int64_t>(blk) * 2 + stamp_copy(st)) * kCopy +
+                                                        (z * kE + row) * kE + x0));
+        const float rq[4] = {rv.x, rv.y, rv.z, rv.w}, pq[4] = {pv.x, pv.y, pv.z, pv.w};
+        unsigned sv = 0u, bb = 0u;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float4 rv = __ldg(reinterpret_cast<const float4*>(rs) + q);
-            const float rq[4] = {rv.x, rv.y, rv.z, rv.w};
-            float4 pv = make_float4(INF, INF, INF, INF);
-            if (ps) pv = __ldcg(reinterpret_cast<const float4*>(ps) + q);
-            const float pq[4] = {pv.x, pv.y, pv.z, pv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int x = 4 * q + e;
-                const float r = rq[e], v = pq[e];
-                if (r > 0.0f && r < INF) {
-                    SV |= 1u << x;
-                    rlo = fminf(rlo, r);
-                }
-                const bool b = v < INF && v > bprev;
-                if (b) {
-                    B |= 1u << x;
-                    mn0 = fminf(mn0, v);
-                }
-                row[x] = b ? -v : v;
+        for (int e = 0; e < 4; ++e) {
+            if (rq[e] > 0.0f && rq[e] < INF) {
+                sv |= 1u << (x0 + e);
+                rlo = fminf(rlo, rq[e]);
             }
+            const float v = band_value(pq[e], bprev);
+            if (sgn(v)) bb |= 1u << (x0 + e);
+            smin = min(smin, sbits(v));
+            S.psi[hx(x0 + e, row, z)] = v;
         }
 #pragma unroll
-        for (int x = 0; x < 32; ++x) S.psi[rb + x] = row[x];
-        S.band[t] = B;
-        S.solv[t] = SV;
-        S.upd[t] = 0u;
+        for (int o = 1; o < 8; o <<= 1) {
+            sv |= __shfl_xor_sync(kFull, sv, o);
+            bb |= __shfl_xor_sync(kFull, bb, o);
+        }
+        if ((lane & 7) == 0) {
+            S.solv[z * kE + row] = sv;
+            S.band[z * kE + row] = bb;
+        }
     }
+    uint4* mk = reinterpret_cast<uint4*>(S.mark + t * kE);        // row t's marks
+    mk[0] = mk[1] = make_uint4(0u, 0u, 0u, 0u);
     // ---- the ghost layer (Alg. 5): the neighbours' boundary layers as of the end
     // of restart k-1, with their Upsilon masks; thread t loads face-local (a, c) =
-    // (lane, warp) of every face.  A ghost node is band when it lies above the
-    // previous bound or the neighbour lowered it in restart k-1.
-    {
-        const int a = lane, c = warp;
+    // (lane, warp) of every face.  A ghost node is tentative when it lies above the
+    // previous bound or the neighbour lowered it in restart k-1; up to the bound it
+    // is accepted at once.
+    const int a = lane, c = warp;
+    float gv[6];
+    unsigned fire = 0u;
 #pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            float g = INF;
-            unsigned um = 0u;
-            if (nbr[f] >= 0) {
-                const unsigned long long w = S.nst[f];
-                int sl = -1, written = -1;
-                if (w != kUntouched) {
-                    if (stamp_latest(w) >= k) {
-                        written = stamp_other(w);
-                        sl = (written == static_cast<int>(kNever)) ? -1 : (stamp_copy(w) ^ 1);
-                    } else {
-                        written = stamp_latest(w);
-                        sl = stamp_copy(w);
-                    }
-                }
-                if (sl >= 0) {
-                    const int64_t cb = static_cast<int64_t>(nbr[f]) * 2 + sl;
-                    g = __ldcg(P.copy + cb * kCopy + nbr_off(f, a, c));
-                    if (written == k - 1) um = __ldcg(P.ups + (cb * 6 + (f ^ 1)) * 32 + c);
+    for (int f = 0; f < 6; ++f) {
+        gv[f] = INF;
+        unsigned um = 0u;
+        if (nbr[f] >= 0) {
+            const unsigned long long w = S.nst[f];
+            int sl = -1, written = -1;
+            if (w != kUntouched) {
+                if (stamp_latest(w) >= k) {
+                    written = stamp_other(w);
+                    sl = (written == static_cast<int>(kNever)) ? -1 : (stamp_copy(w) ^ 1);
+                } else {
+                    written = stamp_latest(w);
+                    sl = stamp_copy(w);
                 }
             }
-            const bool gb = g < INF && (((um >> a) & 1u) || g > bprev);
-            S.psi[ghost_h(f, a, c)] = gb ? -g : g;
-            const unsigned gw = __ballot_sync(kFull, gb);
-            if (lane == 0) S.gband[f][c] = gw;
-            if (gb) mn0 = fminf(mn0, g);
+            if (sl >= 0) {
+                const int64_t cb = static_cast<int64_t>(nbr[f]) * 2 + sl;
+                gv[f] = __ldcg(P.copy + cb * kCopy + nbr_off(f, a, c));
+                if (written == k - 1) um = __ldcg(P.ups + (cb * 6 + (f ^ 1)) * 32 + c);
+            }
+        }
+        const bool tent = gv[f] < INF && (((um >> a) & 1u) || gv[f] > bprev);
+        const bool take = tent && gv[f] <= bound;
+        S.psi[ghost_h(f, a, c)] = tent && !take ? -gv[f] : gv[f];
+        if (take) {
+            smin = min(smin, sbits(-gv[f]));
+            fire |= 1u << f;
         }
     }
-    mn0 = warp_min_nn(mn0);
-    rlo = warp_min_nn(rlo);
-    if (lane == 0) {
-        if (mn0 < INF) atomicMin(&S.mslot[0], __float_as_uint(mn0));
-        if (rlo < INF) atomicMin(&S.wmin, __float_as_uint(rlo));
+    {
+        const float m = warp_min_nn(smin < 0 ? fabsf(__int_as_float(smin)) : INF);
+        rlo = warp_min_nn(rlo);
+        if (lane == 0) {
+            if (m < INF) atomicMin(&S.mn[0], sbits(-m));
+            if (rlo < INF) atomicMin(&S.wmin, __float_as_uint(rlo));
+        }
     }
     __syncthreads();
-    const float w = P.window * __uint_as_float(S.wmin);
+    const unsigned SV = S.solv[t];
+    unsigned nacc = __popc(fire), nsolve = 0u, nupd = 0u;
+    int fb = 0;
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+        // the node next to an accepted ghost node, if it lies above it
+        const int w = (f & 1) ? kE - 1 : 0;
+        const int node = f < 2 ? (c * kE + a) * kE + w : f < 4 ? (c * kE + w) * kE + a : (w * kE + c) * kE + a;
+        const int h = hx(node & 31, (node >> 5) & 31, node >> 10);
+        if (((fire >> f) & 1u) && gv[f] < fabsf(S.psi[h])) S.mark[node] = 1;
+    }
+    const float w = 1.5f * P.window * __uint_as_float(S.wmin);
     const float tau = P.tau;
+    int stages = 0, wave = 0;
+    __syncthreads();
 
-    // ---- rounds (Alg. 4), thread mapping of round_row; lanes 0..5 of warp w also
-    // hold the ghost row c = w of face f = lane
-    const int r = round_row(warp, lane);
-    const int ry = r & 31, rz = r >> 5;
-    const unsigned sv = S.solv[r];
-    const bool gowner = lane < 6;
-    unsigned gbw = gowner ? S.gband[lane][warp] : 0u;
-    unsigned short* wl = S.wl[warp];
-    const unsigned lt = (1u << lane) - 1u;
-    int rounds = 0, par = 0, fb = 0;
-    unsigned nacc = 0u, nsolve = 0u, nupd = 0u;
-    for (int j = 0;; ++j) {
-        const float mn = __uint_as_float(S.mslot[j % 3]);
+    for (;;) {
+        const int m0 = S.mn[stages & 1];
+        const float mn = m0 < 0 ? fabsf(__int_as_float(m0)) : INF;
         if (!(mn < INF) || !(mn <= bound)) break;          // band empty, or its minimum above the bound
-        if (++rounds > kRoundCap) {
+        if (++stages > kRoundCap) {
             if (t == 0) atomicOr(&P.ctrl->status, kStRoundCap);
             break;
         }
-        if (t == 0) S.mslot[(j + 2) % 3] = INFB;         // last read at the start of round j - 1
         const float thr = fminf(mn + w, bound);
-        float kmin = INF;
-        // accept (Remove_Min of a window) of this warp's rows
-        const unsigned bw = S.band[r];
-        unsigned aw = 0u;
+        // ---- tentative nodes of the row up to thr: to be solved (a fixed node only
+        // passes its value on), and the smallest above it
+        smin = 0x7fffffff;
+        unsigned take = 0u;
         {
-            const unsigned nzl = __ballot_sync(kFull, bw != 0u);
-            const int most = __reduce_max_sync(kFull, static_cast<unsigned>(__popc(bw)));
-            if (__popc(nzl) < most) {
-                for (unsigned q = nzl; q; q &= q - 1) {
-                    const int L = __ffs(q) - 1;
-                    const unsigned wL = __shfl_sync(kFull, bw, L);
-                    bool ac = false;
-                    if ((wL >> lane) & 1u) {
-                        const int h = hx(lane, (warp + L) & 31, L);
-                        const float v = fabsf(S.psi[h]);
-                        if (!(thr < v)) {
-                            S.psi[h] = v;
-                            ac = true;
-                        } else {
-                            kmin = fminf(kmin, v);
-                        }
-                    }
-                    const unsigned a = __ballot_sync(kFull, ac);
-                    if (lane == L) aw = a;
-                }
-            } else {
-                const int hb = hx(0, ry, rz);
-                for (unsigned m = bw; m; m &= m - 1) {
-                    const int x = __ffs(m) - 1;
-                    const float v = fabsf(S.psi[hb + x]);
-                    if (!(thr < v)) {
-                        S.psi[hb + x] = v;
-                        aw |= 1u << x;
-                    } else {
-                        kmin = fminf(kmin, v);
-                    }
-                }
+            unsigned gone = 0u;
+            for (unsigned m = S.band[t]; m; m &= m - 1) {
+                const int x = __ffs(m) - 1;
+                const float q = S.psi[rb + x], v = fabsf(q);
+                if (!sgn(q)) gone |= 1u << x;                    // accepted since
+                else if (v <= thr) take |= 1u << x;
+                else smin = min(smin, sbits(-v));
             }
+            if (take | gone) S.band[t] &= ~(take | gone);
         }
-        S.band[r] = bw & ~aw;
-        S.acc[par][r] = aw;
-        nacc += __popc(aw);
-        // the ghost rows, row by row across the lanes
-        {
-            unsigned ga = 0u;
-            for (unsigned q = __ballot_sync(kFull, gbw != 0u); q; q &= q - 1) {
-                const int L = __ffs(q) - 1;
-                const unsigned wL = __shfl_sync(kFull, gbw, L);
-                bool ac = false;
-                if ((wL >> lane) & 1u) {
-                    const int h = ghost_h(L, lane, warp);
-                    const float v = fabsf(S.psi[h]);
-                    if (!(thr < v)) {
-                        S.psi[h] = v;
-                        ac = true;
-                    } else {
-                        kmin = fminf(kmin, v);
-                    }
-                }
-                const unsigned a = __ballot_sync(kFull, ac);
-                if (lane == L) ga = a;
-            }
-            if (gowner) {
-                gbw &= ~ga;
-                S.gacc[par][lane][warp] = ga;
-                nacc += __popc(ga);
-            }
-        }
-        __syncthreads();
-        // neighbours of the accepted nodes (Alg. 2) in this row: x +- 1 by shifts,
-        // the rows at y +- 1 and z +- 1, and the ghost faces at the block's edges
-        unsigned Cw = (aw << 1) | (aw >> 1);
-        Cw |= (ry > 0) ? S.acc[par][r - 1] : S.gacc[par][2][rz];
-        Cw |= (ry < 31) ? S.acc[par][r + 1] : S.gacc[par][3][rz];
-        Cw |= (rz > 0) ? S.acc[par][r - 32] : S.gacc[par][4][ry];
-        Cw |= (rz < 31) ? S.acc[par][r + 32] : S.gacc[par][5][ry];
-        Cw |= (S.gacc[par][0][rz] >> ry) & 1u;
-        Cw |= ((S.gacc[par][1][rz] >> ry) & 1u) << 31;
-        Cw &= sv;
-        // this warp's candidates -> its list (position = exclusive prefix over the
-        // lanes, then bit order), solved kWL at a time by the warp's lanes
-        float smin = INF;
-        {
-            const int cnt = __popc(Cw);
-            int incl = cnt;
+        // ---- waves
+        for (;; ++wave) {
+            // the row's marks -> the list
+            {
+                const uint4 q0 = mk[0], q1 = mk[1];
+                const unsigned wd[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+                const bool marked = (wd[0] | wd[1] | wd[2] | wd[3] | wd[4] | wd[5] | wd[6] | wd[7]) != 0u;
+                if (__any_sync(kFull, marked || take != 0u)) {    // (most planes are away from the front)
+                    unsigned todo = 0u;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int total = __shfl_sync(kFull, incl, 31);
-            const int base = incl - cnt;
-            if (lane == 0) nsolve += static_cast<unsigned>(total);
-            if (total > 0) {
-                const unsigned nzl = __ballot_sync(kFull, Cw != 0u);
-                const bool by_rows = __popc(nzl) < static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(cnt)));
-                for (int done = 0; done < total; done += kWL) {
-                    const int lim = done + kWL;
-                    if (by_rows) {
-                        for (unsigned q = nzl; q; q &= q - 1) {
-                            const int L = __ffs(q) - 1;
-                            const unsigned wL = __shfl_sync(kFull, Cw, L);
-                            const int bL = __shfl_sync(kFull, base, L);
-                            if ((wL >> lane) & 1u) {
-                                const int pos = bL + __popc(wL & lt);
-                                if (pos >= done && pos < lim)
-                                    wl[pos - done] = static_cast<unsigned short>(round_row(warp, L) * 32 + lane);
-                            }
-                        }
-                    } else {
-                        int pos = base;
-                        for (unsigned m = Cw; m; m &= m - 1, ++pos)
-                            if (pos >= done && pos < lim)
-                                wl[pos - done] = static_cast<unsigned short>(r * 32 + __ffs(m) - 1);
+                    for (int i = 0; i < 8; ++i)                   // (bytes 0 or 1 -> 4 bits)
+                        todo |= ((wd[i] * 0x01020408u) >> 24) << (4 * i);
+                    todo = (todo & SV) | take;
+                    const int cnt = __popc(todo);
+                    int incl = cnt;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(kFull, incl, o);
+                        if (lane >= o) incl += v;
                     }
-                    __syncwarp();
-                    const int n = min(kWL, total - done);
-                    for (int i = lane; i < n; i += 32) solve_node(P, S, blk, wl[i], tau, fb, smin, nupd);
-                    __syncwarp();
+                    const int total = __shfl_sync(kFull, incl, 31);
+                    int at = 0;
+                    if (lane == 0 && total > 0) at = atomicAdd(&S.count[wave & 1], total);
+                    at = __shfl_sync(kFull, at, 0) + incl - cnt;
+                    if (at + cnt <= kCap) {
+                        if (marked) mk[0] = mk[1] = make_uint4(0u, 0u, 0u, 0u);
+                        if (cnt) prefetch_l1(rr + t * kE);        // (the row's h/F: 128 bytes)
+                        for (unsigned m = todo; m; m &= m - 1)
+                            S.list[at++] = static_cast<unsigned short>(t * 32 + __ffs(m) - 1);
+                        take = 0u;
+                    } else {
+                        // no room: the row's nodes wait for a later wave
+                        for (; at < kCap; ++at) S.list[at] = 0xffffu;
+                    }
                 }
             }
+            __syncthreads();
+            const int n = min(S.count[wave & 1], kCap);
+            if (n == 0) break;
+            if (t == 0) S.count[(wave + 1) & 1] = 0;           // (read in the wave before this one)
+            for (int base = 32 * warp; base < n; base += kT) {
+                const unsigned entry = base + lane < n ? S.list[base + lane] : 0xffffu;
+                const bool val = entry != 0xffffu;
+                nsolve += val ? 1u : 0u;
+                const int node = val ? static_cast<int>(entry) : 0;
+                const float r = __ldg(rr + node);
+                const int x = node & 31, row = node >> 5, yy = row & 31, zz = row >> 5;
+                float* ps = S.psi + hx(x, yy, zz);
+                volatile const float* pv = ps;
+                const bool live = val && r > 0.0f && r < INF;
+                const float cur = pv[0], cc = fabsf(cur);
+                const float nv[6] = {pv[-1], pv[1], pv[-kH], pv[kH], pv[-kH * kH], pv[kH * kH]};
+                const float mx = axis_min(nv[0], nv[1]), my = axis_min(nv[2], nv[3]), mz = axis_min(nv[4], nv[5]);
+                float a0, a1, a2;
+                sort3(mx, my, mz, a0, a1, a2);
+                const bool go = live && a0 < INF;
+                const float xn = root_fast(a0, a1, a2, r, go, tau, fb);
+                const bool imp = go && xn < cc;
+                const float v = imp ? xn : cc;
+                const bool prop = val && (imp || sgn(cur)) && !(thr < v);
+                if (imp || prop) *const_cast<volatile float*>(ps) = prop ? v : -v;
+                if (imp && !prop) {
+                    smin = min(smin, sbits(-v));
+                    atomicOr(&S.band[row], 1u << x);
+                }
+                nupd += imp ? 1u : 0u;
+                nacc += prop ? 1u : 0u;
+                // mark the neighbours above the accepted value
+                unsigned char* mp = S.mark + node;
+                if (prop && v < fabsf(nv[0]) && x > 0) mp[-1] = 1;
+                if (prop && v < fabsf(nv[1]) && x < 31) mp[1] = 1;
+                if (prop && v < fabsf(nv[2]) && yy > 0) mp[-32] = 1;
+                if (prop && v < fabsf(nv[3]) && yy < 31) mp[32] = 1;
+                if (prop && v < fabsf(nv[4]) && zz > 0) mp[-1024] = 1;
+                if (prop && v < fabsf(nv[5]) && zz < 31) mp[1024] = 1;
+            }
+            __syncthreads();
         }
-        // the next band minimum: of the kept band and of the lowered values
-        {
-            const float v = warp_min_nn(fminf(kmin, smin));
-            if (lane == 0 && v < INF) atomicMin(&S.mslot[(j + 1) % 3], __float_as_uint(v));
-        }
+        if (t == 0) S.mn[stages & 1] = 0x7fffffff;          // (this stage's was in the other slot)
+        const float m = warp_min_nn(smin < 0 ? fabsf(__int_as_float(smin)) : INF);
         __syncthreads();
-        par ^= 1;
+        if (lane == 0 && m < INF) atomicMin(&S.mn[stages & 1], sbits(-m));
+        __syncthreads();
     }
-    if (gowner) S.gband[lane][warp] = gbw;
 
     // ---- statistics of the march
     {
@@ -428,71 +362,72 @@ __device__ void march32(const Params& P, Smem& S, int32_t blk, int k, float bpre
         const unsigned s_ = __reduce_add_sync(kFull, nsolve);
         const int f_ = __reduce_add_sync(kFull, fb);
         if (lane == 0) {
-            atomicAdd(&P.ctrl->r_accepted, static_cast<unsigned long long>(a_));
-            atomicAdd(&P.ctrl->r_updates, static_cast<unsigned long long>(u_));
-            atomicAdd(&P.ctrl->r_solves, static_cast<unsigned long long>(s_));
+            if (a_) atomicAdd(&P.ctrl->r_accepted, static_cast<unsigned long long>(a_));
+            if (u_) atomicAdd(&P.ctrl->r_updates, static_cast<unsigned long long>(u_));
+            if (s_) atomicAdd(&P.ctrl->r_solves, static_cast<unsigned long long>(s_));
             if (f_) atomicAdd(&P.ctrl->r_fallbacks, static_cast<unsigned long long>(f_));
+            if (u_) S.any = 1u;
         }
-        if (t == 0) atomicAdd(&P.ctrl->r_rounds, static_cast<unsigned long long>(rounds));
+        if (t == 0) atomicAdd(&P.ctrl->r_rounds, static_cast<unsigned long long>(stages));
     }
-
-    // ---- write the other copy when the march lowered a value (thread t: row t),
-    // with the Upsilon masks of its faces; list the neighbours across faces with a
-    // lowered node
-    const int y = lane, z = warp, rb = hx(0, y, z);
-    const unsigned U = S.upd[t];
-    const bool lowered = __syncthreads_or(U != 0u) != 0;
-    if (lowered) {
-        const int ns = (st == kUntouched) ? 0 : (stamp_copy(st) ^ 1);
-        const int64_t cb = static_cast<int64_t>(blk) * 2 + ns;
+    __syncthreads();
+    const bool any = S.any != 0u;
+    // ---- Upsilon, per face: the nodes lowered in this march (against the copy it
+    // started from) that lie below the neighbour's node beyond the face; a tentative
+    // ghost node is pending only if it lies below the block's own node
+    const int ns = (st == kUntouched) ? 0 : (stamp_copy(st) ^ 1);
+    const int64_t cb = static_cast<int64_t>(blk) * 2 + ns;
+    {
+        float old[6];
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+            old[f] = INF;
+            // (offset of the block's own face layer: the one its neighbour across it mirrors)
+            if (any && st != kUntouched)
+                old[f] = __ldcg(P.copy + (static_cast<int64_t>(blk) * 2 + stamp_copy(st)) * kCopy + nbr_off(f ^ 1, a, c));
+        }
+        unsigned np = 0u, fm = 0u;
+        for (unsigned m = S.band[t]; m; m &= m - 1) np += sgn(S.psi[rb + __ffs(m) - 1]) ? 1u : 0u;
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+            const int h = ghost_h(f, a, c), d = f < 2 ? 1 : f < 4 ? kH : kH * kH;
+            const float g = S.psi[h], v = fabsf(S.psi[h + ((f & 1) ? -d : d)]);
+            np += sgn(g) && fabsf(g) < v ? 1u : 0u;
+            const unsigned m = __ballot_sync(kFull, any && v < old[f] && v < fabsf(g));
+            if (any && lane == 0) P.ups[(cb * 6 + f) * 32 + c] = m;
+            if (m) fm |= 1u << f;
+        }
+        np = __reduce_add_sync(kFull, np);
+        if (lane == 0 && np) atomicAdd(&S.pend, np);
+        if (lane == 0 && fm) atomicOr(&S.facemask, static_cast<int>(fm));
+    }
+    // ---- write the other copy when the march lowered a value
+    if (any) {
         float* dst = P.copy + cb * kCopy;
-        float v[32];
-#pragma unroll
-        for (int x = 0; x < 32; ++x) v[x] = fabsf(S.psi[rb + x]);
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            reinterpret_cast<float4*>(dst + (z * kE + y) * kE)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2],
-                                                                               v[4 * q + 3]);
-        dst[kX0 + z * kE + y] = v[0];
-        dst[kX31 + z * kE + y] = v[31];
-        unsigned* um = P.ups + cb * 6 * 32;
-        const unsigned w0 = __ballot_sync(kFull, U & 1u), w1 = __ballot_sync(kFull, (U >> 31) & 1u);
-        unsigned fm = 0u;
-        if (lane == 0) {
-            um[0 * 32 + z] = w0;
-            um[1 * 32 + z] = w1;
-            um[2 * 32 + z] = U;                                  // the y = 0 row of plane z
-            fm |= (w0 ? 1u : 0u) | (w1 ? 2u : 0u) | (U ? 4u : 0u);
+#pragma unroll 4
+        for (int i = 0; i < 8; ++i) {
+            const int row = 4 * i + (lane >> 3), x0 = 4 * (lane & 7);
+            const float* q = S.psi + hx(x0, row, z);
+            *reinterpret_cast<float4*>(dst + (z * kE + row) * kE + x0) =
+                make_float4(fabsf(q[0]), fabsf(q[1]), fabsf(q[2]), fabsf(q[3]));
         }
-        if (lane == 31) {
-            um[3 * 32 + z] = U;                                  // the y = 31 row
-            fm |= U ? 8u : 0u;
-        }
-        if (warp == 0) {
-            um[4 * 32 + y] = U;                                  // plane z = 0, row y
-            fm |= U ? 16u : 0u;
-        }
-        if (warp == 31) {
-            um[5 * 32 + y] = U;
-            fm |= U ? 32u : 0u;
-        }
-        if (fm) atomicOr(&S.facemask, static_cast<int>(fm));
-        __syncthreads();
+        dst[kX0 + z * kE + y] = fabsf(S.psi[rb]);
+        dst[kX31 + z * kE + y] = fabsf(S.psi[rb + kE - 1]);
         // (no fence: nobody reads this copy before the grid barrier that ends the restart)
         if (t == 0)
             P.stamp[blk] = make_stamp(k, st == kUntouched ? static_cast<int>(kNever) : stamp_latest(st), ns);
     }
+    __syncthreads();
     // ---- activation for restart k+1 (A of Alg. 4/5, C of Alg. 4)
-    const bool pending = __syncthreads_or(S.band[t] != 0u || (t < 192 && S.gband[t >> 5][t & 31] != 0u)) != 0;
     if (t == 0) {
-        if (pending && grow) enqueue(P, k, blk);
-        const int fm = S.facemask;
-        for (int f = 0; f < 6; ++f)
-            if (((fm >> f) & 1) && nbr[f] >= 0) enqueue(P, k, nbr[f]);
         // publish: the block's restart-k march has finished (read by early marches
         // of its neighbours; the CTA barriers above put every thread's writes before it)
         __threadfence();
         st_release(P.done + blk, k);
+        if (S.pend != 0u && grow) enqueue(P, k, blk);
+        const int fm = S.facemask;
+        for (int f = 0; f < 6; ++f)
+            if (((fm >> f) & 1) && nbr[f] >= 0) enqueue(P, k, nbr[f]);
     }
 }
 

@@ -64,3 +64,27 @@ def test_rough_speeds_and_barriers(eik, orc, dims, precision):
                     assert np.max(np.abs(psi[fin].astype(np.float64) - ref[fin])) <= 1e-5 * ref[fin].max(), (v, edge)
                 base = psi.copy() if base is None else base
                 assert np.array_equal(psi, base), (v, edge)
+
+
+def test_block32_lists_overflow_and_mixed_blocks(eik, orc):
+    """32^3 blocks where a wave's nodes are many (one stage spans the whole block: infinite stride, wide window)
+    and where they are few, rough speeds, ragged grid of 2x2x2 blocks: the 8^3 result bit for bit."""
+    dims = (45, 37, 52)
+    h = synth.grid_h(dims)
+    u = synth.uniform(577, 2, 2 * int(np.prod(dims)))
+    n = int(np.prod(dims))
+    F = (10.0 ** (2.0 * u[:n] - 1.0)).reshape(dims[::-1])
+    F[(u[n:] < 0.05).reshape(dims[::-1])] = 0.0
+    F[0, 0, 0] = F[31, 31, 31] = 1.0
+    F = F.astype(np.float32)
+    with eik.Solver(dims, h, np.ascontiguousarray(F), "fp32") as S:
+        S.add_sources([[0.0, 0.0, 0.0], [31 * h, 31 * h, 31 * h]])
+        S.solve(2 * h, block_dim=8)
+        base = S.result()
+        ref = orc.fmm(F.astype(np.float64), h, [[0.0, 0.0, 0.0], [31 * h, 31 * h, 31 * h]])
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isfinite(base), fin)
+        assert np.max(np.abs(base[fin].astype(np.float64) - ref[fin])) <= 1e-5 * ref[fin].max()
+        for stride, window in ((2.0, 2.0), (4.0, 4.0), (1.0, 1e-3), (math.inf, 1e6), (math.inf, 2.0)):
+            S.solve(stride * h, block_dim=32, window=window)
+            assert np.array_equal(S.result(), base), (stride, window)
