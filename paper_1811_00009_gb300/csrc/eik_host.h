@@ -27,15 +27,16 @@ inline int cell_nodes(double s, double h, int n, int out[2]) {
     return (out[1] == out[0]) ? 1 : 2;
 }
 
-// CTAs of a restart loop over 8^3 bricks, at most per_sm on each of sms SMs.  A
-// small grid's front keeps few warps busy, and the idle ones only poll and crowd
-// the schedulers: ms of a 2h solve with 1, 2, 3 CTAs per SM (GRF speeds, one
-// GB300): 64^3 0.62, 0.64, 0.66; 160^3 2.07, 2.14, 2.24; 200^3 2.80, 2.76, 2.93;
-// 256^3 4.73, 4.24, 4.57; 320^3 7.8, 6.4, 6.7; 400^3 13.4, 10.3, 10.3; 640^3 50.4,
-// 36.2, 34.6.  16^3 blocks (a CTA each) take all.
-inline int restart_loop_ctas(int per_sm, int sms, int64_t nbricks, int block_dim) {
-    const int want = (block_dim == 16 || nbricks > 100000) ? per_sm : (nbricks > 12288 ? 2 : 1);
-    return std::min(per_sm, want) * sms;
+// CTAs of a restart loop over 8^3 bricks on each SM, at most per_sm.  A small grid's
+// front keeps few warps busy, and the idle ones only poll and crowd the schedulers;
+// with fewer CTAs a thread also gets more registers (k_restart_loop is built for each
+// count).  ms of a 2h solve with 1, 2, 3 CTAs per SM (GRF speeds, one GB300): 64^3
+// 0.59, 0.66, 0.70; 160^3 2.14, 2.29, 2.44; 200^3 2.71, 2.71, 2.92; 256^3 4.58, 4.16,
+// 4.52; 320^3 7.6, 6.2, 6.6; 400^3 13.1, 10.1, 10.2; 480^3 23.4, 17.3, 17.0; 640^3
+// 50.9, 36.7, 35.3.  16^3 blocks (a CTA each) take all.
+inline int restart_loop_per_sm(int per_sm, int64_t nbricks, int block_dim) {
+    const int want = (block_dim == 16 || nbricks > 150000) ? per_sm : (nbricks > 12288 ? 2 : 1);
+    return std::min(per_sm, want);
 }
 
 // Brick geometry of one grid inside a launch's brick index space.

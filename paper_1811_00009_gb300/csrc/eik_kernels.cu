@@ -337,9 +337,11 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_group_l
 
 // The restart loop of 8^3 blocks; MIXED: of a schedule whose restarts may also
 // have 16^3 blocks (learned, random).  (A template: with march16 in the loop the
-// compiler has fewer registers for march8.)
-template <typename T, bool MIXED>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(T) == 4 ? 3 : 1) k_restart_loop(const __grid_constant__ LoopParams<T> P) {
+// compiler has fewer registers for march8, 1.5 % at 1024^3.)  RES: CTAs on each SM,
+// by the size of the grid; with one a thread has up to 255 registers instead of 80:
+// 32^3 0.43 -> 0.40 ms, 128^3 with barriers 4.70 -> 4.54, 160^3 2.51 -> 2.44.
+template <typename T, bool MIXED, int RES>
+__global__ void __launch_bounds__(kWarps * 32, RES) k_restart_loop(const __grid_constant__ LoopParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_arrived;
@@ -771,34 +773,43 @@ size_t loop_smem_bytes() {
 }
 
 // Fixed schedules: 8^3 blocks (0) and 16^3 blocks (1); schedules that mix them (2).
+// kind 0: 8^3 blocks, 1: 16^3 blocks, 2: both; res: CTAs on each SM
+template <typename T, int RES>
+const void* loop_kernel_res(int kind) {
+    return kind == 2 ? reinterpret_cast<const void*>(k_restart_loop<T, true, RES>)
+                     : reinterpret_cast<const void*>(k_restart_loop<T, false, RES>);
+}
+
 template <typename T>
-const void* loop_kernel(int kind) {
-    return kind == 1   ? reinterpret_cast<const void*>(k_group_loop<T>)
-           : kind == 2 ? reinterpret_cast<const void*>(k_restart_loop<T, true>)
-                       : reinterpret_cast<const void*>(k_restart_loop<T, false>);
+const void* loop_kernel(int kind, int res) {
+    if (kind == 1) return reinterpret_cast<const void*>(k_group_loop<T>);
+    if (sizeof(T) == 8 || res == 1) return loop_kernel_res<T, 1>(kind);
+    return res == 2 ? loop_kernel_res<T, sizeof(T) == 4 ? 2 : 1>(kind) : loop_kernel_res<T, sizeof(T) == 4 ? 3 : 1>(kind);
 }
 
 template <typename T>
 cudaError_t loop_occupancy(int* blocks_per_sm) {
     const size_t smem = loop_smem_bytes<T>();
+    const int top = sizeof(T) == 4 ? 3 : 1;
     *blocks_per_sm = 1 << 20;
-    for (int kind = 0; kind < 3; ++kind) {
-        const void* f = loop_kernel<T>(kind);
-        int n = 0;
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kWarps * 32, smem);
-        if (e != cudaSuccess) return e;
-        *blocks_per_sm = std::min(*blocks_per_sm, n);
-    }
+    for (int kind = 0; kind < 3; ++kind)
+        for (int res = kind == 1 ? top : 1; res <= top; ++res) {
+            const void* f = loop_kernel<T>(kind, res);
+            int n = 0;
+            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+            if (e == cudaSuccess && res == top) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kWarps * 32, smem);
+            if (e != cudaSuccess) return e;
+            if (res == top) *blocks_per_sm = std::min(*blocks_per_sm, n);
+        }
     return cudaSuccess;
 }
 
 template <typename T>
-cudaError_t launch_restart_loop(const LoopParams<T>& P, int grid, cudaStream_t s) {
+cudaError_t launch_restart_loop(const LoopParams<T>& P, int per_sm, int sms, cudaStream_t s) {
     LoopParams<T> copy = P;
     void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel(loop_kernel<T>(P.gdone != nullptr ? 1 : P.groups ? 2 : 0), dim3(grid), dim3(kWarps * 32), args,
-                                       loop_smem_bytes<T>(), s);
+    return cudaLaunchCooperativeKernel(loop_kernel<T>(P.gdone != nullptr ? 1 : P.groups ? 2 : 0, per_sm), dim3(per_sm * sms),
+                                       dim3(kWarps * 32), args, loop_smem_bytes<T>(), s);
 }
 
 #define EIKG_INSTANTIATE(T)                                                                                     \
@@ -819,7 +830,7 @@ cudaError_t launch_restart_loop(const LoopParams<T>& P, int grid, cudaStream_t s
                                                const void*, int, int32_t*, int64_t, Ctrl*, int32_t*, cudaStream_t); \
     template size_t loop_smem_bytes<T>();                                                                        \
     template cudaError_t loop_occupancy<T>(int*);                                                                \
-    template cudaError_t launch_restart_loop<T>(const LoopParams<T>&, int, cudaStream_t);
+    template cudaError_t launch_restart_loop<T>(const LoopParams<T>&, int, int, cudaStream_t);
 
 EIKG_INSTANTIATE(float)
 EIKG_INSTANTIATE(double)

@@ -45,7 +45,7 @@ cudaError_t launch_result(const T*, const unsigned long long*, T*, int, int, int
 template <typename T>
 cudaError_t loop_occupancy(int*);
 template <typename T>
-cudaError_t launch_restart_loop(const LoopParams<T>&, int, cudaStream_t);
+cudaError_t launch_restart_loop(const LoopParams<T>&, int, int, cudaStream_t);
 }  // namespace eikg
 
 namespace {
@@ -289,7 +289,7 @@ eik_status eik_solve_noalloc(const int32_t dims[3], double h, const float* F, in
         L.nmax = std::max(nx, std::max(ny, nz));
         L.seed = 0;
         if (P.loop_events[0]) NA_CK(cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[0]), st));
-        NA_CK(eikg::launch_restart_loop<float>(L, eikh::restart_loop_ctas(per_sm, sms, L.nbricks, 8), st));
+        NA_CK(eikg::launch_restart_loop<float>(L, eikh::restart_loop_per_sm(per_sm, L.nbricks, 8), sms, st));
         if (P.loop_events[1]) NA_CK(cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[1]), st));
     }
     if (nfix > 0) NA_CK(eikg::launch_restore_r<float>(nfix, d_fb, d_fp, d_saved, rr, st));

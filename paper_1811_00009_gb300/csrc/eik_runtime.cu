@@ -53,7 +53,7 @@ size_t loop_smem_bytes();
 template <typename T>
 cudaError_t loop_occupancy(int*);
 template <typename T>
-cudaError_t launch_restart_loop(const LoopParams<T>&, int, cudaStream_t);
+cudaError_t launch_restart_loop(const LoopParams<T>&, int, int, cudaStream_t);
 }  // namespace eikg
 
 using eikg::kBrick;
@@ -680,7 +680,7 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         }
         if (P.loop_events[0]) EIK_CK(c, cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[0]), s));
         EIK_CK(c, eikg::launch_restart_loop<T>(
-            L, eikh::restart_loop_ctas(c->loop_per_sm, c->sms, c->nbricks, P.block_dim), s));
+            L, eikh::restart_loop_per_sm(c->loop_per_sm, c->nbricks, P.block_dim), c->sms, s));
         if (P.loop_events[1]) EIK_CK(c, cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[1]), s));
     }
     if (nfix > 0)
@@ -1072,9 +1072,9 @@ eik_status eik_slab_restart(eik_ctx* c, int64_t* pending) {
     if (!c) return fail(nullptr, EIK_EINVAL, "eik_slab_restart: ctx is NULL");
     if (!c->slab_running) return fail(c, EIK_ESTATE, "eik_slab_restart: no sharded solve begun (eik_slab_begin)");
     EIK_CK(c, cudaMemsetAsync(&c->ctrl->done, 0, sizeof(int32_t), c->stream));
-    const int ctas = eikh::restart_loop_ctas(c->loop_per_sm, c->sms, c->nbricks, 8);
-    if (c->prec == EIK_FP32) EIK_CK(c, eikg::launch_restart_loop<float>(c->lp_f, ctas, c->stream));
-    else EIK_CK(c, eikg::launch_restart_loop<double>(c->lp_d, ctas, c->stream));
+    const int per_sm = eikh::restart_loop_per_sm(c->loop_per_sm, c->nbricks, 8);
+    if (c->prec == EIK_FP32) EIK_CK(c, eikg::launch_restart_loop<float>(c->lp_f, per_sm, c->sms, c->stream));
+    else EIK_CK(c, eikg::launch_restart_loop<double>(c->lp_d, per_sm, c->sms, c->stream));
     return slab_pending(c, pending);
 }
 

@@ -88,3 +88,21 @@ def test_block32_lists_overflow_and_mixed_blocks(eik, orc):
         for stride, window in ((2.0, 2.0), (4.0, 4.0), (1.0, 1e-3), (math.inf, 1e6), (math.inf, 2.0)):
             S.solve(stride * h, block_dim=32, window=window)
             assert np.array_equal(S.result(), base), (stride, window)
+
+
+@pytest.mark.parametrize("dims", [(184, 184, 184), (192, 189, 184), (448, 432, 408)])
+def test_launch_sizes(eik, dims):
+    """The 8^3 loop as built for one, two and three blocks of threads an SM (grids on both sides of the first line and
+    above the second), a fixed and a random schedule (8^3 and 16^3 restarts in turn): the 16^3 loop's result bit for bit."""
+    import torch
+    h = synth.grid_h(dims)
+    g = torch.Generator(device="cuda").manual_seed(dims[0])
+    F = (10.0 ** (torch.rand(dims[::-1], generator=g, device="cuda") - 0.5)).float()
+    with eik.Solver(dims, h, F, "fp32") as S:
+        S.add_sources([[0.0, 0.0, 0.0], [0.5 * dims[0] * h, 0.7 * dims[1] * h, 0.4 * dims[2] * h]])
+        S.solve(2.0 * h, block_dim=16)
+        base = S.result().copy()
+        assert np.all(np.isfinite(base))
+        for kw in (dict(block_dim=8), dict(schedule=eik.EIK_SCHED_RANDOM, seed=5)):
+            S.solve(2.0 * h, **kw)
+            assert np.array_equal(S.result(), base), kw
