@@ -34,11 +34,11 @@ METRIC = "Eikonal Mpoints/s at 512^3/1024^3 + HBM roofline %; learned vs fixed s
 ALGO_BYTES_PER_POINT = {"fp32": 8, "fp64": 16}      # read F once + write psi once
 KERNELS_PER_SOLVE = 4                                # gather_r, init_sources, restart_loop, restore_r
 # DRAM bytes and warp instructions per node of k_restart_loop (fixed stride 2h, 8^3 blocks, FP32) from an ncu
-# capture of the same workload family at 512^3 (dram__bytes_read.sum + dram__bytes_write.sum = 9.387 GB +
-# 4.636 GB; smsp__inst_executed.sum = 23.517 G over 512^3 nodes), scaled to the launch by its node count;
+# capture of the same workload family at 512^3 (dram__bytes_read.sum + dram__bytes_write.sum = 7.642 GB +
+# 4.339 GB; smsp__inst_executed.sum = 15.425 G over 512^3 nodes), scaled to the launch by its node count;
 # profiles/k_restart_loop_c4_512_fixed2h.md gives the command.
-NCU_TRAFFIC_PER_NODE = {"fp32": (9.436e9 + 4.657e9) / 512 ** 3}
-NCU_INST_PER_NODE = {"fp32": 23.852e9 / 512 ** 3}
+NCU_TRAFFIC_PER_NODE = {"fp32": (7.642e9 + 4.339e9) / 512 ** 3}
+NCU_INST_PER_NODE = {"fp32": 15.425e9 / 512 ** 3}
 ISSUE_PER_SM_CYCLE = 4          # warp schedulers per SM, one warp instruction per cycle each
 
 

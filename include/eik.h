@@ -138,9 +138,10 @@ typedef struct {
                                network under the learned schedule (8 for restarts 1-2), else the edge
                                eik_autotune chose for the context, else 8 */
     int32_t schedule;       /* eik_schedule */
-    double window;          /* acceptance window factor omega: each march round accepts every band
-                               point within omega * h / F_max(block) of the band minimum
-                               (0 = default 2; 1/sqrt(3) is the smallest increment of Alg. 3) */
+    double window;          /* window factor omega: each stage of a march settles the band points within
+                               1.5 * omega * h / F_max(block) of the band minimum (0 = default 2; 32^3
+                               blocks: the same; 1/sqrt(3) is the smallest increment of Alg. 3).  psi does
+                               not depend on it */
     double fallback_tau;    /* FP32 mode: fall back to double when D < tau * k * (h/F)^2 (0 = default 1/8) */
     int64_t max_restarts;   /* restart cap (0 = default 1 << 24); reaching it returns EIK_ETIMEOUT */
     int32_t log_restarts;   /* non-zero: record per-restart statistics (eik_restart_log) */
@@ -166,7 +167,7 @@ typedef struct {
     int64_t solves;         /* upwind solves (Alg. 3 calls) */
     int64_t updates;        /* solves that lowered psi (Alg. 2 accepted updates) */
     int64_t fallbacks;      /* FP32 roots recomputed in double */
-    int64_t rounds;         /* acceptance rounds over all marches */
+    int64_t rounds;         /* stages over all marches */
     double device_ms;       /* device time of the restart loop (%globaltimer) */
     double final_bound;     /* bound of the last restart */
     int32_t status;         /* eik_status of the device run */
@@ -415,7 +416,7 @@ typedef struct {
     int64_t solves;         /* upwind solves (Alg. 3), summed over grids */
     int64_t updates;        /* solves that lowered psi */
     int64_t fallbacks;      /* FP32 roots recomputed in double */
-    int64_t rounds;         /* acceptance rounds */
+    int64_t rounds;         /* stages over all marches */
     double device_ms;       /* device time of the launch (%globaltimer) */
     int32_t status;         /* eik_status of the device run */
     int32_t ctas;           /* CTAs of the launch */

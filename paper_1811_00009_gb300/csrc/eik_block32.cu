@@ -11,7 +11,8 @@
 // Data layout in HBM (one grid): blocks b = (bz*NBY + by)*NBX + bx of 32^3
 // nodes, node p = (z*32 + y)*32 + x; the ragged last block of each axis is
 // padded with barrier nodes.
-//   rr[b][32768]          h/F (+inf: barrier or padding, -1: fixed source node)
+//   rr[b][32768]          h/F; -inf (barrier, padding of the 8^3 bricks), -1 (fixed
+//                         source node) or +inf (beyond the bricks): not solved
 //   copy[b][2][34816]     two copies of the block's psi: 32768 interior values,
 //                         then the x = 0 and x = 31 layers (1024 each, index
 //                         z*32 + y) stored contiguously for the neighbours
@@ -56,7 +57,7 @@ struct Params {
     int32_t* list[kRing];              // work lists by ring slot; entries not yet written are -1
     int32_t* done;                     // per block: last restart whose march of it finished (-1: none)
     Ctrl* ctrl;
-    float window;                      // omega: acceptance window = omega * min(h/F) over the block
+    float window;                      // omega: a stage spans 1.5 * omega * min(h/F) over the block
     float tau;                         // FP64 root fallback threshold
     double width;                      // width_band
     int64_t max_restarts;

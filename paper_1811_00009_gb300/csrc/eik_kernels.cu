@@ -1,6 +1,7 @@
 // Device kernels of libeik for one grid: the block-based restarted
 // narrow-band fast marching method (J. Yang 2018, Alg. 6 with Algs. 1-5) on
-// sm_103a.  The march itself (Algs. 2-5) is in eik_march.cuh.
+// sm_103a.  The marches themselves (Algs. 2-5) are in eik_march8.cuh and
+// eik_march16.cuh.
 //
 // The restart loop of Alg. 6 runs in one cooperative persistent kernel with
 // one grid-wide barrier per restart; the exchange step (Alg. 5) is fused into

@@ -1,26 +1,9 @@
-// Device code shared by the restart-loop kernels (one grid, eik_kernels.cu;
-// many grids, eik_batch.cu): the upwind root of Alg. 3, the per-warp shared
-// memory of a march, and March_Narrow_Band (Alg. 4 with Algs. 2, 3 and the
-// ghost exchange of Alg. 5).
-//
-// One warp marches one 8x8x8 block (a "brick").  The brick's psi, h/F and its
-// six ghost faces sit in shared memory; lane L loads and writes back the two
-// x-rows (y = L & 7, z = 2*(L >> 3) + {0, 1}) and face-local nodes 2L, 2L+1 of
-// each ghost face.  The band (Sec. 2.1 BAND set) is a list of halo indices
-// shared by the warp; a band node's value carries its sign bit set in shared
-// memory so that any lane can tell a tentative value from an accepted (KNOWN)
-// one with one load.
-//
-// Ordered extraction (Alg. 4) is done in rounds: each round accepts every band
-// node with psi <= min(m + w, bound), m the band minimum, w = omega * min(h/F)
-// over the brick; the accepted nodes' neighbours (Alg. 2) come from shifting a
-// halo bit vector of the accepted nodes, are compacted into a list and
-// re-solved (Alg. 3) 32 at a time.  A lowered node rejoins the band, so an
-// accepted node can be refreshed later exactly as a KNOWN_NEW node of the
-// paper can.  With w = 0 this is the paper's one-node-at-a-time order.
-//
-// The rest of the file is the restart loop's shared machinery: the work-list
-// ring, the per-warp grid barrier and the early marches of the next restart.
+// Device code shared by the restart-loop kernels (one grid, eik_kernels.cu; many
+// grids, eik_batch.cu): the upwind root of Alg. 3 and the restart loop's machinery
+// -- the ring of work lists, the grid barrier that CTAs arrive at and poll as one,
+// and the early marches of the next restart while they wait.  The marches of one
+// block (Alg. 4) are in eik_march8.cuh (a warp per 8^3 block), eik_march16.cuh (a
+// CTA per 16^3 block) and eik_block32.cu (a CTA per 32^3 block).
 #pragma once
 
 #include "eik_internal.cuh"
@@ -109,20 +92,21 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 // is non-decreasing in x and non-increasing in every v_i: a value v_i >= x
 // adds nothing, which is the growth rule of Alg. 3.
 //
-// The result returned is the value x of the working precision at which
-// G_fl(x) comes nearest r^2 from either side (root_search), G_fl being G
+// In double precision the marches take the exact root rounded to the nearest
+// double (root_fast in eik_march8.cuh).  In single precision they take the value x
+// at which G_fl(x) comes nearest r^2 from either side (root_search), G_fl being G
 // evaluated with round-to-nearest operations in a fixed order (largest term
-// first; no contraction).  Every operation in G_fl is monotone in its
-// operands, so G_fl keeps both monotonicities, and the returned root is then
-// a monotone function of (a, b, c): a neighbour that is lower can never give
-// a higher root.  The discrete solution is the
+// first; no contraction); every operation in G_fl is monotone in its operands, so
+// G_fl keeps both monotonicities.  Either root is a monotone function of
+// (a, b, c): a neighbour that is lower can never give a higher root.  The discrete
+// solution is the
 // greatest fixed point of psi_p = min(psi_p, root_p(neighbours)) below the
 // initial values (+inf off the sources); iterations of a monotone map from
 // above reach that one fixed point in any order, so psi does not depend on
 // the stride, the schedule, the block edge or the order of the marches, bit
 // for bit.
 //
-// The search starts from a fast estimate of the root, written without
+// The search in single precision starts from a fast estimate, written without
 // cancellation: with k admitted values,
 //   x = v_1 + (sum_i (v_i - v_1) + sqrt(D)) / k,
 //   D = k r^2 - sum_{i<j} (v_i - v_j)^2          (Lagrange's identity),
