@@ -42,6 +42,14 @@ constexpr int kWarps = 8;          // warps per CTA of the restart loop (one bri
 constexpr long long kWaitPolls = 1ll << 22;   // polls (naps of 32 ns to 4 us) before a wait gives up: seconds
 constexpr int kRing = 4;           // work lists in flight: restart k's, k+1's, k+2's (early k+1 marches), k-1's (being cleared)
 
+// Word arrays that a solve sets to one value each (k_reset).
+struct ResetList {
+    int32_t* p[7];
+    int64_t n[7];
+    int32_t value[7];
+    int count;
+};
+
 constexpr unsigned long long kUntouched = ~0ull;   // stamp of a brick no march has written
 constexpr unsigned kNever = 0x7fffffffu;           // "other copy never written"
 

@@ -544,6 +544,29 @@ __global__ void k_restore_r(int nfix, const int32_t* __restrict__ fix_b, const i
     if (t < nfix) rr[static_cast<int64_t>(fix_b[t]) * kBrick + fix_p[t]] = saved_r[t];
 }
 
+// The per-brick state of a new solve: one launch for all the arrays instead of four
+// to seven memsets, with 16-byte stores (the arrays are allocations of their own).
+// With the host's tables in one copy each and the control block read back by the
+// stream, 32^3 395 -> 384 us a call, 97x61x130 1.29 -> 1.27 ms: launches, not bytes.
+__global__ void k_reset(const __grid_constant__ ResetList R) {
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t width = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int a = 0; a < R.count; ++a) {
+        const int32_t v = R.value[a];
+        const int64_t n4 = R.n[a] >> 2;
+        int4* p4 = reinterpret_cast<int4*>(R.p[a]);
+        for (int64_t i = t; i < n4; i += width) p4[i] = make_int4(v, v, v, v);
+        if (t < (R.n[a] & 3)) R.p[a][4 * n4 + t] = v;
+    }
+}
+
+cudaError_t launch_reset(const ResetList& R, cudaStream_t s) {
+    int64_t most = 1;
+    for (int a = 0; a < R.count; ++a) most = std::max(most, R.n[a] / 4 + 1);
+    k_reset<<<static_cast<int>(std::min<int64_t>((most + 255) / 256, 152 * 8)), 256, 0, s>>>(R);
+    return cudaGetLastError();
+}
+
 // h/F of selected nodes (brick, node) for the host's source set-up.
 template <typename T>
 __global__ void k_gather_r(int n, const int32_t* __restrict__ nb_b, const int32_t* __restrict__ nb_p,

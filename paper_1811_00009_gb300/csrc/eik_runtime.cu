@@ -52,6 +52,7 @@ template <typename T>
 size_t loop_smem_bytes();
 template <typename T>
 cudaError_t loop_occupancy(int*);
+cudaError_t launch_reset(const ResetList&, cudaStream_t);
 template <typename T>
 cudaError_t launch_restart_loop(const LoopParams<T>&, int, int, cudaStream_t);
 }  // namespace eikg
@@ -113,6 +114,7 @@ struct eik_ctx {
     int sms = 0;
     eik_params params{};
     eikg::Ctrl host_ctrl{};
+    eikg::Ctrl* h_ctrl = nullptr;  // pinned: the control block as the solve in flight leaves it
     std::string err;
     // part of a grid sharded in z across GPUs (eik_slab_*): the brick planes this context owns, and the
     // restart loop's parameters between the restarts of a sharded solve
@@ -173,6 +175,7 @@ void free_all(eik_ctx* c) {
         if (p) cudaFree(p);
     if (c->h_err) cudaFreeHost(c->h_err);
     if (c->h_gather) cudaFreeHost(c->h_gather);
+    if (c->h_ctrl) cudaFreeHost(c->h_ctrl);
 }
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
@@ -344,6 +347,8 @@ eik_status eik_create(eik_ctx** out, const int32_t dims[3], double h, const void
             return bail(st, m);
         }
     }
+    e = cudaHostAlloc(reinterpret_cast<void**>(&c->h_ctrl), sizeof(eikg::Ctrl), cudaHostAllocDefault);
+    if (e != cudaSuccess) return bail(EIK_ENOMEM, std::string("eik_create: control block: ") + cudaGetErrorString(e));
     int per_sm = 0;
     e = (c->prec == EIK_FP32) ? eikg::loop_occupancy<float>(&per_sm) : eikg::loop_occupancy<double>(&per_sm);
     if (e != cudaSuccess || per_sm < 1)
@@ -499,10 +504,13 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
     eikh::source_candidates(c->src.data(), nsrc, c->nx, c->ny, c->slab ? c->nz_all : c->nz, c->h, geo, cand,
                             c->slab ? c->zoff : 0, c->nz);
     const int nc = static_cast<int>(cand.size());
-    std::vector<int32_t> cb(nc), cp(nc);
+    // (tables that go to the device together are laid out on the host as there: one
+    // copy: a small solve is bound by the number of calls)
+    const size_t table = align_up(nc * 4);
+    std::vector<char> cbp(2 * table);
     for (int t = 0; t < nc; ++t) {
-        cb[t] = cand[t].b;
-        cp[t] = cand[t].p;
+        reinterpret_cast<int32_t*>(cbp.data())[t] = cand[t].b;
+        reinterpret_cast<int32_t*>(cbp.data() + table)[t] = cand[t].p;
     }
     // scratch: candidate tables, then the fixed-node tables
     const size_t need = align_up(nc * 4) * 2 + align_up(nc * 8) + align_up(nc * 4) * 4 + align_up(nc * 8) +
@@ -534,9 +542,32 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
             EIK_CK(c, cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->d_gather), c->h_gather, 0));
             c->gather_cap = nc;
         }
-        EIK_CK(c, cudaMemcpyAsync(d_cb, cb.data(), nc * 4, cudaMemcpyHostToDevice, s));
-        EIK_CK(c, cudaMemcpyAsync(d_cp, cp.data(), nc * 4, cudaMemcpyHostToDevice, s));
+        EIK_CK(c, cudaMemcpyAsync(d_cb, cbp.data(), cbp.size(), cudaMemcpyHostToDevice, s));
         EIK_CK(c, eikg::launch_gather_r<T>(nc, d_cb, d_cp, static_cast<const T*>(c->rr), c->d_gather, s));
+    }
+    // ---- Alg. 1 for every brick: untouched (psi = +inf) unless it holds fixed nodes
+    const bool groups = (P.block_dim == 16) || (P.schedule != EIK_SCHED_FIXED);
+    const size_t nb = static_cast<size_t>(c->nbricks);
+    {
+        eikg::ResetList R{};
+        auto add = [&](void* p, int64_t words, int32_t value) {
+            R.p[R.count] = static_cast<int32_t*>(p);
+            R.n[R.count] = words;
+            R.value[R.count++] = value;
+        };
+        const int64_t b = c->nbricks, g = c->ngroups;
+        add(c->stamp, 2 * b, -1);
+        add(c->queued, eikg::kRing * b, -1);
+        add(c->lists, eikg::kRing * b, -1);            // empty entries are -1
+        add(c->done, b, 0);
+        if (groups) {
+            add(c->qgroup, eikg::kRing * g, -1);
+            add(c->glists, eikg::kRing * g, -1);
+            add(c->gdone, g, 0);
+        }
+        EIK_CK(c, eikg::launch_reset(R, s));
+    }
+    if (nc > 0) {
         EIK_CK(c, cudaStreamSynchronize(s));
         for (int t = 0; t < nc; ++t) cr[t] = reinterpret_cast<volatile double*>(c->h_gather)[t];
     }
@@ -551,17 +582,9 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         }
         enq.swap(own);
     }
-    const bool groups = (P.block_dim == 16) || (P.schedule != EIK_SCHED_FIXED);
     std::vector<int32_t> genq;
     if (groups) genq = eikh::groups_of(enq, geo, c->GX, c->GY, 0);
     const int nfix = static_cast<int>(uf.size());
-    std::vector<int32_t> fb(nfix), fp(nfix);
-    std::vector<double> fv(nfix);
-    for (int t = 0; t < nfix; ++t) {
-        fb[t] = uf[t].b;
-        fp[t] = uf[t].p;
-        fv[t] = uf[t].v;
-    }
     c->d_fix_b = reinterpret_cast<int32_t*>(carve(nfix * 4));
     c->d_fix_p = reinterpret_cast<int32_t*>(carve(nfix * 4));
     double* d_fv = reinterpret_cast<double*>(carve(nfix * 8));
@@ -571,24 +594,19 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
     c->d_saved_r = carve(nfix * sizeof(T));
     c->nfix = nfix;
     if (nfix > 0) {
-        EIK_CK(c, cudaMemcpyAsync(c->d_fix_b, fb.data(), nfix * 4, cudaMemcpyHostToDevice, s));
-        EIK_CK(c, cudaMemcpyAsync(c->d_fix_p, fp.data(), nfix * 4, cudaMemcpyHostToDevice, s));
-        EIK_CK(c, cudaMemcpyAsync(d_fv, fv.data(), nfix * 8, cudaMemcpyHostToDevice, s));
-        EIK_CK(c, cudaMemcpyAsync(d_sb, sb.data(), sb.size() * 4, cudaMemcpyHostToDevice, s));
-        EIK_CK(c, cudaMemcpyAsync(d_enq, enq.data(), enq.size() * 4, cudaMemcpyHostToDevice, s));
-        if (!genq.empty())
-            EIK_CK(c, cudaMemcpyAsync(d_genq, genq.data(), genq.size() * 4, cudaMemcpyHostToDevice, s));
-    }
-    // ---- Alg. 1 for every brick: untouched (psi = +inf) unless it holds fixed nodes
-    const size_t nb = static_cast<size_t>(c->nbricks);
-    EIK_CK(c, cudaMemsetAsync(c->stamp, 0xFF, nb * sizeof(unsigned long long), s));
-    EIK_CK(c, cudaMemsetAsync(c->queued, 0xFF, eikg::kRing * nb * sizeof(int32_t), s));
-    EIK_CK(c, cudaMemsetAsync(c->lists, 0xFF, eikg::kRing * nb * sizeof(int32_t), s));     // empty entries are -1
-    EIK_CK(c, cudaMemsetAsync(c->done, 0, nb * sizeof(int32_t), s));
-    if (groups) {
-        EIK_CK(c, cudaMemsetAsync(c->qgroup, 0xFF, eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
-        EIK_CK(c, cudaMemsetAsync(c->glists, 0xFF, eikg::kRing * static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
-        EIK_CK(c, cudaMemsetAsync(c->gdone, 0, static_cast<size_t>(c->ngroups) * sizeof(int32_t), s));
+        const char* base = reinterpret_cast<const char*>(c->d_fix_b);
+        std::vector<char> up(static_cast<const char*>(c->d_saved_r) - base);
+        auto host = [&](const void* dev) { return up.data() + (static_cast<const char*>(dev) - base); };
+        for (int t = 0; t < nfix; ++t) {
+            reinterpret_cast<int32_t*>(host(c->d_fix_b))[t] = uf[t].b;
+            reinterpret_cast<int32_t*>(host(c->d_fix_p))[t] = uf[t].p;
+            reinterpret_cast<double*>(host(d_fv))[t] = uf[t].v;
+        }
+        auto put = [&](const int32_t* dev, const std::vector<int32_t>& v) { std::copy(v.begin(), v.end(), reinterpret_cast<int32_t*>(host(dev))); };
+        put(d_sb, sb);
+        put(d_enq, enq);
+        put(d_genq, genq);
+        EIK_CK(c, cudaMemcpyAsync(c->d_fix_b, up.data(), up.size(), cudaMemcpyHostToDevice, s));
     }
     if (nfix > 0)
         EIK_CK(c, eikg::launch_init_sources<T>(nfix, c->d_fix_b, c->d_fix_p, d_fv, static_cast<int>(sb.size()), d_sb,
@@ -901,6 +919,7 @@ eik_status eik_solve_async(eik_ctx* c, const eik_params* params) {
         c->last_edge = 8;
     }
     if (st != EIK_OK) return st;
+    EIK_CK(c, cudaMemcpyAsync(c->h_ctrl, c->ctrl, sizeof(eikg::Ctrl), cudaMemcpyDeviceToHost, c->stream));
     c->in_flight = true;
     c->solved = false;
     return EIK_OK;
@@ -911,8 +930,7 @@ eik_status eik_wait(eik_ctx* c, eik_stats* stats) {
     if (!c->in_flight) return fail(c, EIK_ESTATE, "eik_wait: no solve in flight");
     c->in_flight = false;
     EIK_CK(c, cudaStreamSynchronize(c->stream));
-    eikg::Ctrl H{};
-    EIK_CK(c, cudaMemcpy(&H, c->ctrl, sizeof(H), cudaMemcpyDeviceToHost));
+    const eikg::Ctrl H = *c->h_ctrl;
     c->host_ctrl = H;
     c->last_nr = H.k;
     eik_status st = EIK_OK;
