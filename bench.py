@@ -32,7 +32,7 @@ if ROOT not in sys.path:
 
 METRIC = "Eikonal Mpoints/s at 512^3/1024^3 + HBM roofline %; learned vs fixed stride"
 ALGO_BYTES_PER_POINT = {"fp32": 8, "fp64": 16}      # read F once + write psi once
-KERNELS_PER_SOLVE = 4                                # gather_r, init_sources, restart_loop, restore_r
+KERNELS_PER_SOLVE = 5                                # gather_r, reset, init_sources, restart_loop, restore_r
 # DRAM bytes and warp instructions per node of k_restart_loop (fixed stride 2h, 8^3 blocks, FP32) from an ncu
 # capture of the same workload family at 512^3 (dram__bytes_read.sum + dram__bytes_write.sum = 7.642 GB +
 # 4.339 GB; smsp__inst_executed.sum = 15.425 G over 512^3 nodes), scaled to the launch by its node count;
