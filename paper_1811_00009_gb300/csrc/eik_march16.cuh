@@ -428,6 +428,28 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
             }
         }
     }
+    // A schedule that mixes block edges (it keeps the brick list) may march the next
+    // restart brick by brick: a tentative node across an inner face of the group that
+    // lies below the brick's own node is then a ghost this brick has to see.  Nothing
+    // else would tell it, since the node's brick accepts it without lowering it.  (Not
+    // counted in the band: the node's own brick counts it.)
+    bool across = false;
+    if (G.lists & 1u) {
+        auto pending = [&](int h, int d) {
+            const T g = S.psi[h + d];
+            return sgn(g) && vlt(vabs(g), vabs(S.psi[h]));
+        };
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int h = hbase + kUp * s;
+            across = across || pending(h + (wx ? 0 : 7), wx ? -1 : 1);
+            if (y == (wy ? 0 : 7))
+                for (int x = 0; x < 8; ++x) across = across || pending(h + x, wy ? -kH16 : kH16);
+            if (z0 + s == (wz ? 0 : 7))
+                for (int x = 0; x < 8; ++x) across = across || pending(h + x, wz ? -kUp : kUp);
+        }
+        across = __any_sync(kFull, across);
+    }
     low = __any_sync(kFull, low);
     nt = __reduce_add_sync(kFull, nt);
     if (lane == 0 && nt) atomicAdd(&S.pend[warp], nt);
@@ -461,8 +483,9 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
         // restart (a reader that sees the new stamp takes the other copy).
         if (lane == 6) P.stamp[b] = make_stamp(k, own < 0 ? static_cast<int>(kNever) : stamp_latest(ms), ns);
     }
-    // ---- activation for restart k+1 (A of Alg. 4/5, C of Alg. 4; none across the group's own faces, whose masks are 0)
-    if (lane == 6 && S.pend[warp] != 0u && grow) enqueue_next(P, G, k, b);
+    // ---- activation for restart k+1 (A of Alg. 4/5, C of Alg. 4; across the group's own faces, whose masks are 0, only
+    // for tentative nodes, see above: the accepted ones have reached the other brick in this march)
+    if (lane == 6 && (S.pend[warp] != 0u || across) && grow) enqueue_next(P, G, k, b);
     if (lane < 6 && S.mask[warp][lane] != 0ull) {
         const int ax = lane >> 1, w1 = (lane & 1) ? 1 : -1;
         const int32_t nb = brick(2 * gx + wx + (ax == 0 ? w1 : 0), 2 * gy + wy + (ax == 1 ? w1 : 0),
