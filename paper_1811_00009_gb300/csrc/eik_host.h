@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <vector>
 
@@ -160,6 +161,38 @@ inline void first_active(const std::vector<FixNode>& fix, const Bricks& g, std::
     sb.resize(ns);
     enq.resize(ne);
 }
+
+// The tables of a solve's sources on the device, in one allocation: byte offsets of
+// the candidates (brick, node), then of the fixed nodes (brick, node, psi0), the
+// bricks that hold them, the work lists of restart 1 (bricks, groups) and the fixed
+// nodes' saved h/F (elem bytes each), every table on a 256-byte line.
+struct SolveTables {
+    size_t cand_b, cand_p, fix_b, fix_p, fix_v, src_b, enq, genq, saved, end;
+};
+inline SolveTables solve_tables(size_t nc, size_t nfix, size_t nsb, size_t nenq, size_t ngenq, size_t elem) {
+    SolveTables t;
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += (bytes + 255) & ~size_t(255);
+        return at;
+    };
+    t.cand_b = take(nc * 4);
+    t.cand_p = take(nc * 4);
+    t.fix_b = take(nfix * 4);
+    t.fix_p = take(nfix * 4);
+    t.fix_v = take(nfix * 8);
+    t.src_b = take(nsb * 4);
+    t.enq = take(nenq * 4);
+    t.genq = take(ngenq * 4);
+    t.saved = take(nfix * elem);
+    t.end = o;
+    return t;
+}
+// Room for the tables of nc candidates, whichever of them become fixed nodes: at most
+// nc fixed nodes in as many bricks, and up to 7 bricks of restart 1 each
+// (first_active_into), in as many groups.
+inline size_t solve_tables_room(size_t nc, size_t elem) { return solve_tables(nc, nc, nc, 7 * nc, 7 * nc, elem).end; }
 
 // The checks every solve entry point applies to eik_params (the learned
 // schedule's weights are the caller's to check): nullptr if the parameters are

@@ -506,15 +506,13 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
     const int nc = static_cast<int>(cand.size());
     // (tables that go to the device together are laid out on the host as there: one
     // copy: a small solve is bound by the number of calls)
-    const size_t table = align_up(nc * 4);
-    std::vector<char> cbp(2 * table);
+    const eikh::SolveTables ct = eikh::solve_tables(nc, 0, 0, 0, 0, sizeof(T));
+    std::vector<char> cbp(ct.fix_b);
     for (int t = 0; t < nc; ++t) {
-        reinterpret_cast<int32_t*>(cbp.data())[t] = cand[t].b;
-        reinterpret_cast<int32_t*>(cbp.data() + table)[t] = cand[t].p;
+        reinterpret_cast<int32_t*>(cbp.data() + ct.cand_b)[t] = cand[t].b;
+        reinterpret_cast<int32_t*>(cbp.data() + ct.cand_p)[t] = cand[t].p;
     }
-    // scratch: candidate tables, then the fixed-node tables
-    const size_t need = align_up(nc * 4) * 2 + align_up(nc * 8) + align_up(nc * 4) * 4 + align_up(nc * 8) +
-                        align_up(nc * sizeof(T)) + 4096;
+    const size_t need = eikh::solve_tables_room(nc, sizeof(T));
     if (need > c->scratch_cap) {
         if (c->scratch) cudaFree(c->scratch);
         c->scratch = nullptr;
@@ -523,14 +521,8 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         c->scratch_cap = need;
     }
     char* sp = static_cast<char*>(c->scratch);
-    auto carve = [&](size_t bytes) {
-        char* r = sp;
-        sp += align_up(bytes);
-        return r;
-    };
-    int32_t* d_cb = reinterpret_cast<int32_t*>(carve(nc * 4));
-    int32_t* d_cp = reinterpret_cast<int32_t*>(carve(nc * 4));
-    carve(nc * 8);
+    int32_t* d_cb = reinterpret_cast<int32_t*>(sp + ct.cand_b);
+    int32_t* d_cp = reinterpret_cast<int32_t*>(sp + ct.cand_p);
     std::vector<double> cr(nc);
     if (nc > 0) {
         if (nc > c->gather_cap) {
@@ -585,13 +577,15 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
     std::vector<int32_t> genq;
     if (groups) genq = eikh::groups_of(enq, geo, c->GX, c->GY, 0);
     const int nfix = static_cast<int>(uf.size());
-    c->d_fix_b = reinterpret_cast<int32_t*>(carve(nfix * 4));
-    c->d_fix_p = reinterpret_cast<int32_t*>(carve(nfix * 4));
-    double* d_fv = reinterpret_cast<double*>(carve(nfix * 8));
-    int32_t* d_sb = reinterpret_cast<int32_t*>(carve(sb.size() * 4));
-    int32_t* d_enq = reinterpret_cast<int32_t*>(carve(enq.size() * 4));
-    int32_t* d_genq = reinterpret_cast<int32_t*>(carve(genq.size() * 4));
-    c->d_saved_r = carve(nfix * sizeof(T));
+    const eikh::SolveTables ft = eikh::solve_tables(nc, nfix, sb.size(), enq.size(), genq.size(), sizeof(T));
+    if (ft.end > c->scratch_cap) return fail(c, EIK_ECUDA, "source tables larger than their scratch");
+    c->d_fix_b = reinterpret_cast<int32_t*>(sp + ft.fix_b);
+    c->d_fix_p = reinterpret_cast<int32_t*>(sp + ft.fix_p);
+    double* d_fv = reinterpret_cast<double*>(sp + ft.fix_v);
+    int32_t* d_sb = reinterpret_cast<int32_t*>(sp + ft.src_b);
+    int32_t* d_enq = reinterpret_cast<int32_t*>(sp + ft.enq);
+    int32_t* d_genq = reinterpret_cast<int32_t*>(sp + ft.genq);
+    c->d_saved_r = sp + ft.saved;
     c->nfix = nfix;
     if (nfix > 0) {
         const char* base = reinterpret_cast<const char*>(c->d_fix_b);
