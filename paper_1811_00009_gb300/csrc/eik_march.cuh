@@ -93,7 +93,7 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 // adds nothing, which is the growth rule of Alg. 3.
 //
 // In double precision the marches take the exact root rounded to the nearest
-// double (root_fast in eik_march8.cuh).  In single precision they take the value x
+// double (root_fast in eik_root64.cuh).  In single precision they take the value x
 // at which G_fl(x) comes nearest r^2 from either side (root_search), G_fl being G
 // evaluated with round-to-nearest operations in a fixed order (largest term
 // first; no contraction); every operation in G_fl is monotone in its operands, so
@@ -234,6 +234,12 @@ __device__ __forceinline__ T root_near(T x0, T a, T b, T c, T r2) {
         }
     }
     return root_search<T>(x0, a, b, c, r2);
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 // The estimate (with the causality clamps: in exact arithmetic the root is not
