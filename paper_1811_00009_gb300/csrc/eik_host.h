@@ -194,6 +194,13 @@ inline SolveTables solve_tables(size_t nc, size_t nfix, size_t nsb, size_t nenq,
 // (first_active_into), in as many groups.
 inline size_t solve_tables_room(size_t nc, size_t elem) { return solve_tables(nc, nc, nc, 7 * nc, 7 * nc, elem).end; }
 
+// The limit of a solve's device-side waits: the caller's wait_polls, or `preset` for 0.
+// Kernels multiply it by small constants, so it stays far below the type's largest
+// value: 2^56 polls take centuries.
+inline long long wait_limit(int64_t wait_polls, long long preset) {
+    return wait_polls > 0 ? static_cast<long long>(std::min(wait_polls, int64_t(1) << 56)) : preset;
+}
+
 // The checks every solve entry point applies to eik_params (the learned
 // schedule's weights are the caller's to check): nullptr if the parameters are
 // valid, else the message, with the status in *code.

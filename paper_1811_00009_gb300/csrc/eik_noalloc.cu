@@ -282,7 +282,7 @@ eik_status eik_solve_noalloc(const int32_t dims[3], double h, const float* F, in
         L.fallback_tau = P.fallback_tau;
         L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
-        L.wait_limit = P.wait_polls > 0 ? P.wait_polls : eikg::kWaitPolls;
+        L.wait_limit = eikh::wait_limit(P.wait_polls, eikg::kWaitPolls);
         L.sched = EIK_SCHED_FIXED;
         L.mlp = nullptr;
         L.h = h;

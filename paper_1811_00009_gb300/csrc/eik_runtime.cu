@@ -673,7 +673,7 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.width = P.width;
-        L.wait_limit = P.wait_polls > 0 ? P.wait_polls : eikg::kWaitPolls;
+        L.wait_limit = eikh::wait_limit(P.wait_polls, eikg::kWaitPolls);
         L.sched = P.schedule;
         L.mlp = (P.schedule == EIK_SCHED_LEARNED) ? c->d_mlp : nullptr;
         L.h = c->h;
@@ -859,7 +859,7 @@ eik_status queue_solve32(eik_ctx* c, const eik_params& P) {
         EIK_CK(c, eikg::block32_loop(B.NBX, B.NBY, B.NBZ, B.nblk, B.copy, B.ups, B.stamp, B.rr, B.queued, B.lists, B.done,
                                      c->ctrl,
                                      static_cast<float>(P.window), static_cast<float>(P.fallback_tau), P.width,
-                                     P.max_restarts, P.wait_polls > 0 ? P.wait_polls : eikg::kWaitPolls, B.grid, s));
+                                     P.max_restarts, eikh::wait_limit(P.wait_polls, eikg::kWaitPolls), B.grid, s));
         if (P.loop_events[1]) EIK_CK(c, cudaEventRecord(static_cast<cudaEvent_t>(P.loop_events[1]), s));
     }
     if (nfix > 0)
