@@ -39,7 +39,15 @@ constexpr int kSlot = 640;         // values per brick copy
 constexpr int kXF0 = 512;          // offset of the x = 0 face inside a copy
 constexpr int kXF7 = 576;          // offset of the x = 7 face
 constexpr int kWarps = 8;          // warps per CTA of the restart loop (one brick per warp)
-constexpr long long kWaitPolls = 1ll << 22;   // polls (naps of 32 ns to 4 us) before a wait gives up: seconds
+constexpr long long kWaitPolls = 1ll << 22;   // polls (naps of up to kWaitNap) before a wait gives up: seconds
+// Longest naps (ns) between polls: the unit of the limit; at the grid barrier; of a warp
+// that watches its CTA's poller.  Waits with shorter naps take as many more polls
+// (the watchers twice that, so that the poller gives up first).
+constexpr int kWaitNap = 4096;
+constexpr int kBarrierNap = 512;
+constexpr int kWatchNap = 256;
+constexpr int kBarrierPolls = kWaitNap / kBarrierNap;
+constexpr int kWatchPolls = 2 * kWaitNap / kWatchNap;
 constexpr int kRing = 4;           // work lists in flight: restart k's, k+1's, k+2's (early k+1 marches), k-1's (being cleared)
 
 // Word arrays that a solve sets to one value each (k_reset).

@@ -696,10 +696,10 @@ __device__ int wait_or_work(const LoopParams<T>& P, CtaLoop& S, int k, unsigned 
             if (vol(S.stop)) st = 2;
             else if (vol(S.rel) != gen) st = 1;
             else if (vol(S.token) == 0 && atomicCAS(&S.token, 0, 1) == 0) st = 3;
-            else if (it > 8 * P.wait_limit) st = 4;
+            else if (it > kWatchPolls * P.wait_limit) st = 4;
             if (st) break;
             __nanosleep(nap);
-            if (nap < 256) nap <<= 1;
+            if (nap < kWatchNap) nap <<= 1;
         }
         if (st == 3) {
             nap = 32;
@@ -737,12 +737,12 @@ __device__ int wait_or_work(const LoopParams<T>& P, CtaLoop& S, int k, unsigned 
                         break;
                     }
                 }
-                if (it > P.wait_limit) {
+                if (it > kBarrierPolls * P.wait_limit) {
                     st = 4;
                     break;
                 }
                 __nanosleep(nap);
-                if (nap < 512) nap <<= 1;
+                if (nap < kBarrierNap) nap <<= 1;
             }
             __threadfence_block();
             atomicExch(&S.token, 0);
@@ -796,21 +796,22 @@ __device__ int wait_or_group(const LoopParams<T>& P, CtaLoop& S, int k, unsigned
                 const int32_t near[7] = {x, gx > 0 ? x - 1 : -1, gx < P.GX - 1 ? x + 1 : -1, gy > 0 ? x - P.GX : -1,
                                          gy < P.GY - 1 ? x + P.GX : -1, gz > 0 ? x - P.GX * P.GY : -1,
                                          gz < P.GZ - 1 ? x + P.GX * P.GY : -1};
-                long long w = x < 0 ? P.wait_limit + 1 : 0;
-                for (int j = 0; j < 7 && w <= P.wait_limit; ++j) {
+                const long long most = kBarrierPolls * P.wait_limit;
+                long long w = x < 0 ? most + 1 : 0;
+                for (int j = 0; j < 7 && w <= most; ++j) {
                     if (near[j] < 0 || __ldcg(P.qgroup + static_cast<int64_t>(s) * P.ngroups + near[j]) != k) continue;
                     unsigned d = 64;
-                    for (w = 0; ld_acquire(P.gdone + near[j]) < k && w <= P.wait_limit; ++w) {
+                    for (w = 0; ld_acquire(P.gdone + near[j]) < k && w <= most; ++w) {
                         __nanosleep(d);
-                        if (d < 512) d <<= 1;
+                        if (d < kBarrierNap) d <<= 1;
                     }
                 }
-                if (w > P.wait_limit) st = 4;
+                if (w > most) st = 4;
                 break;
             }
-            if (it > P.wait_limit) st = 4;
+            if (it > kBarrierPolls * P.wait_limit) st = 4;
             __nanosleep(nap);
-            if (nap < 512) nap <<= 1;
+            if (nap < kBarrierNap) nap <<= 1;
         }
         if (st == 4) {
             atomicOr(&C->status, kStWaitTimeout);

@@ -27,6 +27,22 @@ def test_limit_leaves_room_for_the_kernels_factors(tmp_path):
         assert preset < f(polls, preset) <= LARGEST // 64
 
 
+def test_shorter_naps_take_more_polls(tmp_path):
+    """A wait with shorter naps than the 4 us the limit counts takes as many more polls, and a warp that watches its CTA's
+    poller waits longer than the poller."""
+    from paper_1811_00009_gb300 import build
+    src, lib = tmp_path / "naps.cpp", tmp_path / "naps.so"
+    src.write_text('#include "eik_internal.cuh"\n'
+                   'extern "C" int unit() { return eikg::kWaitNap; }\n'
+                   'extern "C" int barrier() { return eikg::kBarrierPolls * eikg::kBarrierNap; }\n'
+                   'extern "C" int watch() { return eikg::kWatchPolls * eikg::kWatchNap; }\n')
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-fPIC", "-shared", "-I" + cuda, "-I" + build.CSRC, str(src), "-o", str(lib)],
+                   check=True)
+    L = C.CDLL(str(lib))
+    assert L.unit() == 4096 and L.barrier() >= L.unit() and L.watch() >= 2 * L.barrier()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("kw", [dict(block_dim=8), dict(block_dim=16), dict(block_dim=32), dict(schedule=2, seed=3)],
                          ids=["blocks8", "blocks16", "blocks32", "random"])
