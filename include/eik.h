@@ -364,7 +364,8 @@ eik_status eik_mlp_forward(const float *w, const float *X, int32_t B, float *Y, 
 
 /* eik_mlp_grad -- loss = mean_s (Y[s][act[s]] - tgt[s])^2 and its gradient grad[PARAMS] with respect
  * to w; DEVICE pointers; work holds eik_mlp_work_floats(B) floats owned by the caller.  The sum over
- * samples runs in a fixed order, so the result is deterministic. */
+ * samples runs in a fixed order, so the result is deterministic.  (Work: 1805 floats per 128 samples; 0
+ * for B < 1 and for more samples than an int32_t of floats serves, 152 million, which eik_mlp_grad refuses.) */
 eik_status eik_mlp_grad(const float *w, const float *X, const int32_t *act, const float *tgt, int32_t B,
                         float *grad, float *loss, float *work, void *stream);
 int32_t eik_mlp_work_floats(int32_t B);

@@ -14,6 +14,7 @@
 #include "eik.h"
 #include "eik_mlp.cuh"
 
+#include <cstdint>
 #include <string>
 
 namespace {
@@ -27,11 +28,10 @@ eik_status mlp_fail(eik_status s, const std::string& m) {
     return s;
 }
 
-// workspace floats per sample that eik_mlp_work_floats asks for (the partial sums
-// use less)
-constexpr int kWork = 4 * kHid + 1;
 constexpr int kChunk = 128;            // samples per block of the gradient kernel
 constexpr int kPitch = kChunk + 4;     // row pitch of the sample arrays (float4 rows on different banks)
+
+inline int64_t grad_blocks(int32_t B) { return B > 0 ? (static_cast<int64_t>(B) + kChunk - 1) / kChunk : 0; }
 
 // The weights as the threads read them (the same address in every lane, four at a time).
 struct __align__(16) NetSmem {
@@ -266,7 +266,8 @@ extern "C" {
 const char* eik_mlp_last_error(void) { return g_mlp_err.c_str(); }
 
 int32_t eik_mlp_work_floats(int32_t B) {
-    return B > 0 ? B * kWork + ((B + 255) / 256) * (kParams + 1) : 0;
+    const int64_t n = grad_blocks(B) * (kParams + 1);
+    return n <= INT32_MAX ? static_cast<int32_t>(n) : 0;
 }
 
 eik_status eik_mlp_forward(const float* w, const float* X, int32_t B, float* Y, void* stream) {
@@ -281,8 +282,10 @@ eik_status eik_mlp_forward(const float* w, const float* X, int32_t B, float* Y, 
 eik_status eik_mlp_grad(const float* w, const float* X, const int32_t* act, const float* tgt, int32_t B, float* grad,
                         float* loss, float* work, void* stream) {
     if (!w || !X || !act || !tgt || !grad || !work || B < 1) return mlp_fail(EIK_EINVAL, "eik_mlp_grad: bad argument");
+    if (eik_mlp_work_floats(B) == 0)
+        return mlp_fail(EIK_EINVAL, "eik_mlp_grad: more samples than a work space of 2^31 - 1 floats serves");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int nchunks = (B + kChunk - 1) / kChunk;
+    const int nchunks = static_cast<int>(grad_blocks(B));
     const cudaError_t attr = cudaFuncSetAttribute(k_mlp_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   static_cast<int>(sizeof(GradSmem)));
     if (attr != cudaSuccess) return mlp_fail(EIK_ECUDA, cudaGetErrorString(attr));
