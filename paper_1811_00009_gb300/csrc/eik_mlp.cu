@@ -137,20 +137,6 @@ __device__ __forceinline__ float total(const float* p) {
     return (a0 + a1) + (a2 + a3);
 }
 
-// sum over the block's samples of p[s] q[s] where p[s] is not 0 (q[s] may then be anything)
-__device__ __forceinline__ float dot_taken(const float* p, const float* q) {
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll 8
-    for (int s = 0; s < kChunk; s += 4) {
-        const float4 u = *reinterpret_cast<const float4*>(p + s), v = *reinterpret_cast<const float4*>(q + s);
-        a0 = __fmaf_rn(u.x, u.x != 0.0f ? v.x : 0.0f, a0);
-        a1 = __fmaf_rn(u.y, u.y != 0.0f ? v.y : 0.0f, a1);
-        a2 = __fmaf_rn(u.z, u.z != 0.0f ? v.z : 0.0f, a2);
-        a3 = __fmaf_rn(u.w, u.w != 0.0f ? v.w : 0.0f, a3);
-    }
-    return (a0 + a1) + (a2 + a3);
-}
-
 // Block c: forward, error of the taken action and backpropagated deltas of its
 // samples, then partial[c][p] = their sum for every parameter p (and, for p ==
 // kParams, of the squared errors).  Places without a sample hold zeros, and a sample
@@ -171,8 +157,10 @@ __global__ void __launch_bounds__(kChunk) k_mlp_partial(const float* __restrict_
             S.x[j][t] = x[j];
         }
         hidden(S.net, x, u, v);                                  // u = h1, v = h2
+        // (a hidden value that is not a number makes y and with it dy one, so W3's row of
+        // the action taken is lost either way; the other rows are to keep a zero)
 #pragma unroll
-        for (int j = 0; j < kHid; ++j) S.h1[j][t] = in ? u[j] : 0.0f, S.h2[j][t] = in ? v[j] : 0.0f;
+        for (int j = 0; j < kHid; ++j) S.h1[j][t] = in ? u[j] : 0.0f, S.h2[j][t] = in && v[j] == v[j] ? v[j] : 0.0f;
         const int a = in ? act[s] : 0;
         float y = S.net.b3[a];
 #pragma unroll
@@ -215,7 +203,7 @@ __global__ void __launch_bounds__(kChunk) k_mlp_partial(const float* __restrict_
         for (int j = 0; j < 8; ++j) out[kOffW2 + i * kHid + j0 + j] = acc[j][0] + acc[j][1];
     }
     for (int p = t; p < kHid * kIn; p += kChunk) out[kOffW1 + p] = dot(S.d1[p / kIn], S.x[p % kIn]);       // d1_i x_j
-    for (int p = t; p < kAct * kHid; p += kChunk) out[kOffW3 + p] = dot_taken(S.dy[p / kHid], S.h2[p % kHid]);   // dy_a h2_j
+    for (int p = t; p < kAct * kHid; p += kChunk) out[kOffW3 + p] = dot(S.dy[p / kHid], S.h2[p % kHid]);   // dy_a h2_j
     if (t < kHid) out[kOffB1 + t] = total(S.d1[t]);
     else if (t < 2 * kHid) out[kOffB2 + t - kHid] = total(S.d2[t - kHid]);
     else if (t < 2 * kHid + kAct) out[kOffB3 + t - 2 * kHid] = total(S.dy[t - 2 * kHid]);
