@@ -142,7 +142,10 @@ typedef struct {
                                1.5 * omega * h / F_max(block) of the band minimum (0 = default 2; 32^3
                                blocks: the same; 1/sqrt(3) is the smallest increment of Alg. 3).  psi does
                                not depend on it */
-    double fallback_tau;    /* FP32 mode: fall back to double when D < tau * k * (h/F)^2 (0 = default 1/8) */
+    double fallback_tau;    /* FP32 mode: a root's estimate is taken in double when D < tau * k * (h/F)^2 (0 =
+                               default 1/8).  D >= (h/F)^2 but for rounding, so below tau = 1/3 the marches
+                               make this test (up to tau = 0.33) only for estimates that miss the root by
+                               more than an ulp.  psi does not depend on it */
     int64_t max_restarts;   /* restart cap (0 = default 1 << 24); reaching it returns EIK_ETIMEOUT */
     int32_t log_restarts;   /* non-zero: record per-restart statistics (eik_restart_log) */
     int32_t seed;           /* EIK_SCHED_RANDOM seed */
@@ -167,7 +170,7 @@ typedef struct {
     int64_t accepted;       /* band points accepted (heap pops in Alg. 4), refreshes included */
     int64_t solves;         /* upwind solves (Alg. 3 calls) */
     int64_t updates;        /* solves that lowered psi (Alg. 2 accepted updates) */
-    int64_t fallbacks;      /* FP32 roots recomputed in double */
+    int64_t fallbacks;      /* FP32 roots or their estimates taken in double (see eik_params.fallback_tau) */
     int64_t rounds;         /* stages over all marches */
     double device_ms;       /* device time of the restart loop (%globaltimer) */
     double final_bound;     /* bound of the last restart */
@@ -417,7 +420,7 @@ typedef struct {
     int64_t accepted;       /* band points accepted, summed over grids */
     int64_t solves;         /* upwind solves (Alg. 3), summed over grids */
     int64_t updates;        /* solves that lowered psi */
-    int64_t fallbacks;      /* FP32 roots recomputed in double */
+    int64_t fallbacks;      /* FP32 roots or their estimates taken in double (see eik_params.fallback_tau) */
     int64_t rounds;         /* stages over all marches */
     double device_ms;       /* device time of the launch (%globaltimer) */
     int32_t status;         /* eik_status of the device run */

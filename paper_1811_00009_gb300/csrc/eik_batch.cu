@@ -651,7 +651,6 @@ eik_status batch_queue(eik_batch* b, const std::vector<eik_batch_tile>& tiles, i
         L.ctrl = b->ctrl;
         L.window = P.window;
         L.window_f = static_cast<float>(P.window);
-        L.fallback_tau = P.fallback_tau;
         L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.width = INFINITY;                    // full solves

@@ -201,12 +201,10 @@ struct LoopParams {
     int64_t log_cap;
     double window;             // omega: acceptance window = omega * min(h/F) over the brick
     float window_f;            // omega in single precision (FP32 marches compute the window in float)
-    double fallback_tau;       // FP32: double-precision root when D < tau * k * r^2
-    float tau_f;               // the same in single precision
+    float tau_f;               // FP32: fallback_tau (eik_params), the estimate in double precision when D < tau * k * r^2
     int64_t max_restarts;
     long long wait_limit;      // polls before a wait (barrier, list entry, neighbour march) gives up
     int32_t sched;             // 0 fixed, 1 learned, 2 seeded random (exploration data)
-    int32_t mode_fixed;        // block edge of every restart under the fixed schedule (8 or 16)
     const float* mlp;          // schedule network weights (learned schedule)
     double h;
     int32_t nmax;              // longest grid axis (feature scale)

@@ -791,13 +791,14 @@ cudaError_t launch_slab_import(T* slot, unsigned long long* ups, unsigned long l
     return cudaGetLastError();
 }
 
+// kind: a fixed schedule of 8^3 blocks (0) or of 16^3 blocks (1), a schedule that
+// mixes them (2); res: CTAs on each SM
 template <typename T>
-size_t loop_smem_bytes() {
-    return std::max(sizeof(GroupSmem<T>), sizeof(QueueSmem<T>) * kWarps);
+size_t loop_smem_bytes(int kind) {
+    const size_t group = sizeof(GroupSmem<T>), queues = sizeof(QueueSmem<T>) * kWarps;
+    return kind == 0 ? queues : kind == 1 ? group : std::max(group, queues);
 }
 
-// Fixed schedules: 8^3 blocks (0) and 16^3 blocks (1); schedules that mix them (2).
-// kind 0: 8^3 blocks, 1: 16^3 blocks, 2: both; res: CTAs on each SM
 template <typename T, int RES>
 const void* loop_kernel_res(int kind) {
     return kind == 2 ? reinterpret_cast<const void*>(k_restart_loop<T, true, RES>)
@@ -813,12 +814,12 @@ const void* loop_kernel(int kind, int res) {
 
 template <typename T>
 cudaError_t loop_occupancy(int* blocks_per_sm) {
-    const size_t smem = loop_smem_bytes<T>();
     const int top = sizeof(T) == 4 ? 3 : 1;
     *blocks_per_sm = 1 << 20;
     for (int kind = 0; kind < 3; ++kind)
         for (int res = kind == 1 ? top : 1; res <= top; ++res) {
             const void* f = loop_kernel<T>(kind, res);
+            const size_t smem = loop_smem_bytes<T>(kind);
             int n = 0;
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
             if (e == cudaSuccess && res == top) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kWarps * 32, smem);
@@ -832,8 +833,9 @@ template <typename T>
 cudaError_t launch_restart_loop(const LoopParams<T>& P, int per_sm, int sms, cudaStream_t s) {
     LoopParams<T> copy = P;
     void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel(loop_kernel<T>(P.gdone != nullptr ? 1 : P.groups ? 2 : 0, per_sm), dim3(per_sm * sms),
-                                       dim3(kWarps * 32), args, loop_smem_bytes<T>(), s);
+    const int kind = P.gdone != nullptr ? 1 : P.groups ? 2 : 0;
+    return cudaLaunchCooperativeKernel(loop_kernel<T>(kind, per_sm), dim3(per_sm * sms), dim3(kWarps * 32), args,
+                                       loop_smem_bytes<T>(kind), s);
 }
 
 #define EIKG_INSTANTIATE(T)                                                                                     \
@@ -852,7 +854,6 @@ cudaError_t launch_restart_loop(const LoopParams<T>& P, int per_sm, int sms, cud
                                                int, int, int, void*, cudaStream_t);                              \
     template cudaError_t launch_slab_import<T>(T*, unsigned long long*, unsigned long long*, int, int, int, int,   \
                                                const void*, int, int32_t*, int64_t, Ctrl*, int32_t*, cudaStream_t); \
-    template size_t loop_smem_bytes<T>();                                                                        \
     template cudaError_t loop_occupancy<T>(int*);                                                                \
     template cudaError_t launch_restart_loop<T>(const LoopParams<T>&, int, int, cudaStream_t);
 

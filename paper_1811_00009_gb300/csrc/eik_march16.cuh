@@ -11,7 +11,11 @@
 // A neighbour's value may be read before or after that neighbour's own solve of
 // the wave; either is an upper bound of what it ends with, and as the wave starts
 // with clearing its nodes' queue marks, a neighbour that is lowered queues them
-// again for the next.
+// again for the next.  So may a listed node's h/F be read while another thread's mark
+// (a NaN) stands in its sign word: the node then counts as one that is never solved,
+// passes on the value it has, and is solved in the next wave, since a marked node is
+// always in the next list.  Either way psi ends the same; the counts of solves and
+// accepted nodes depend on the timing.
 //
 // What bounds it: the chain of waves (two of its three latencies are shared-memory
 // round trips) and, with all SMs busy, issue slots.  The march this replaces gave
@@ -313,7 +317,9 @@ __device__ __forceinline__ void march16(const LoopParams<T>& P, const Geo& G, Ma
                 T* ps = S.psi + hq;
                 volatile const T* pv = ps;
                 const T r = vabs(S.rq[hq]);
-                const bool live = val && vlt(r, INF);            // (a fixed node only passes its value on)
+                // (a fixed node only passes its value on, and so does one that is just
+                // being marked for the next wave: r is a NaN)
+                const bool live = val && vlt(r, INF);
                 const T cur = pv[0], c = vabs(cur);
                 const T nv[6] = {pv[-1], pv[1], pv[-kH16], pv[kH16], pv[-kUp], pv[kUp]};
                 const T mx = axis_min(nv[0], nv[1]), my = axis_min(nv[2], nv[3]), mz = axis_min(nv[4], nv[5]);

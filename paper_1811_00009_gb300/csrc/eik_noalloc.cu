@@ -272,14 +272,12 @@ eik_status eik_solve_noalloc(const int32_t dims[3], double h, const float* F, in
         for (int r = 0; r < eikg::kRing; ++r) L.list[r] = lists + r * nb;
         L.early = 1;
         L.groups = 0;                 // 8^3 blocks only: no group work lists
-        L.mode_fixed = 8;
         L.ctrl = ctrl;
         L.log = nullptr;
         L.log_cap = 0;
         L.window = P.window;
         L.window_f = static_cast<float>(P.window);
         L.width = P.width;
-        L.fallback_tau = P.fallback_tau;
         L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.wait_limit = eikh::wait_limit(P.wait_polls, eikg::kWaitPolls);

@@ -49,8 +49,6 @@ cudaError_t block32_result(const float*, const unsigned long long*, float*, int,
 cudaError_t block32_loop(int, int, int, int64_t, float*, unsigned*, unsigned long long*, const float*, int32_t*,
                          int32_t*, int32_t*, Ctrl*, float, float, double, int64_t, long long, int, cudaStream_t);
 template <typename T>
-size_t loop_smem_bytes();
-template <typename T>
 cudaError_t loop_occupancy(int*);
 cudaError_t launch_reset(const ResetList&, cudaStream_t);
 template <typename T>
@@ -663,13 +661,11 @@ eik_status queue_solve(eik_ctx* c, const eik_params& P, bool slab = false) {
         L.GZ = c->GZ;
         L.groups = groups ? 1 : 0;
         L.qgroup = c->qgroup;
-        L.mode_fixed = (P.block_dim == 16) ? 16 : 8;
         L.ctrl = c->ctrl;
         L.log = P.log_restarts ? c->log : nullptr;
         L.log_cap = P.log_restarts ? c->log_cap : 0;
         L.window = P.window;
         L.window_f = static_cast<float>(P.window);
-        L.fallback_tau = P.fallback_tau;
         L.tau_f = static_cast<float>(P.fallback_tau);
         L.max_restarts = P.max_restarts;
         L.width = P.width;
