@@ -157,10 +157,8 @@ __global__ void __launch_bounds__(kChunk) k_mlp_partial(const float* __restrict_
             S.x[j][t] = x[j];
         }
         hidden(S.net, x, u, v);                                  // u = h1, v = h2
-        // (a hidden value that is not a number makes y and with it dy one, so W3's row of
-        // the action taken is lost either way; the other rows are to keep a zero)
 #pragma unroll
-        for (int j = 0; j < kHid; ++j) S.h1[j][t] = in ? u[j] : 0.0f, S.h2[j][t] = in && v[j] == v[j] ? v[j] : 0.0f;
+        for (int j = 0; j < kHid; ++j) S.h1[j][t] = u[j], S.h2[j][t] = v[j];
         const int a = in ? act[s] : 0;
         float y = S.net.b3[a];
 #pragma unroll
@@ -172,7 +170,7 @@ __global__ void __launch_bounds__(kChunk) k_mlp_partial(const float* __restrict_
         for (int q = 0; q < kAct; ++q) S.dy[q][t] = q == a ? dy : 0.0f;
 #pragma unroll
         for (int j = 0; j < kHid; ++j) {
-            v[j] = in ? dy * S.net.w3[a][j] * (1.0f - v[j] * v[j]) : 0.0f;   // d2
+            v[j] = dy * S.net.w3[a][j] * (1.0f - v[j] * v[j]);   // d2
             S.d2[j][t] = v[j];
         }
 #pragma unroll
@@ -181,7 +179,16 @@ __global__ void __launch_bounds__(kChunk) k_mlp_partial(const float* __restrict_
 #pragma unroll
         for (int j = 0; j < kHid; ++j) {
             const float h = S.h1[j][t];
-            S.d1[j][t] = in ? u[j] * (1.0f - h * h) : 0.0f;
+            S.d1[j][t] = u[j] * (1.0f - h * h);
+        }
+        // A hidden value that is not a number makes y and with it dy none either, so W3's
+        // row of the action taken is lost; the other rows multiply it by 0.  (Guarded
+        // where they are stored, the values of all samples took 0.2 us of 53.)
+        if (!in || !(dy == dy)) {
+            for (int j = 0; j < kHid; ++j) {
+                S.h2[j][t] = 0.0f;
+                if (!in) S.h1[j][t] = S.d1[j][t] = S.d2[j][t] = 0.0f;
+            }
         }
     }
     __syncthreads();
